@@ -98,6 +98,60 @@ std::vector<int> dif_positions(const AxisPlan& p) {
   return pos;
 }
 
+// fewest passes after merging neighbours whose product is a supported radix <= max_radix; among
+// equal counts the smallest sum of radices (fewer registers, less arithmetic)
+ExecPlan make_exec_plan(const AxisPlan& a, int max_radix) {
+  ExecPlan e = {};
+  e.n = a.n;
+  auto mergeable = [&](int i) {   // the pairs the kernels have (every pair with a product <= 16 that plans hold)
+    const int ra = a.radix[i], rb = a.radix[i + 1];
+    const bool have = (rb == 2 && ra >= 5 && ra <= 8) || (rb == 3 && (ra == 3 || ra == 5));
+    return have && ra * rb <= max_radix;
+  };
+  const int n = a.nst;
+  int cnt[kMaxStages + 2] = {0}, sum[kMaxStages + 2] = {0};
+  bool two[kMaxStages + 2] = {false};
+  for (int i = n - 1; i >= 0; --i) {
+    cnt[i] = 1 + cnt[i + 1];
+    sum[i] = a.radix[i] + sum[i + 1];
+    if (i + 1 < n && mergeable(i)) {
+      const int c = 1 + cnt[i + 2], s = a.radix[i] * a.radix[i + 1] + sum[i + 2];
+      if (c < cnt[i] || (c == cnt[i] && s < sum[i])) {
+        cnt[i] = c;
+        sum[i] = s;
+        two[i] = true;
+      }
+    }
+  }
+  for (int i = 0; i < n; i += two[i] ? 2 : 1) {
+    ExecPass& p = e.p[e.nst++];
+    p.R = two[i] ? a.radix[i] * a.radix[i + 1] : a.radix[i];
+    p.L = a.blk[i];
+    p.S = p.L / p.R;
+    p.mS = magic(p.S);
+    p.tw = e.ntw;
+    if (p.S > 1) e.ntw += p.L;
+    e.big |= p.R > 8;
+  }
+  if (e.nst == 0) e.p[e.nst++] = ExecPass{1, 1, 1, magic(1), 0};
+  return e;
+}
+
+// exp(2 pi i j r / L) of every pass with S > 1, in the layout of ExecPass::tw
+static std::vector<double2> exec_twiddles(const ExecPlan& e) {
+  std::vector<double2> tw(std::max(1, e.ntw), double2{1.0, 0.0});
+  for (int s = 0; s < e.nst; ++s) {
+    const ExecPass& p = e.p[s];
+    if (p.S == 1) continue;
+    for (int j = 0; j < p.S; ++j)
+      for (int r = 0; r < p.R; ++r) {
+        const double ang = 2.0 * 3.14159265358979323846 * (j * r % p.L) / p.L;
+        tw[p.tw + j * p.R + r] = double2{std::cos(ang), std::sin(ang)};
+      }
+  }
+  return tw;
+}
+
 // complex spherical harmonics, Condon-Shortley phase, l <= 2, unit vector u
 static std::complex<double> ylm(int l, int m, const double u[3]) {
   const double pi = 3.14159265358979323846;
@@ -211,17 +265,25 @@ static int build_k(dks_ctx* ctx, const double kfrac[3], double ecut, const dks_p
   kp.qmax = std::sqrt(qmax2);
   DKS_TRY(upload(&kp.stick_start, sstart.data(), sstart.size()));
   DKS_TRY(upload(&kp.stick_plane, splane.data(), splane.size()));
+  std::vector<int> prow;
+  for (int at : splane) prow.push_back(at / ctx->plane_ld * ctx->plane_ld);
+  std::sort(prow.begin(), prow.end());
+  prow.erase(std::unique(prow.begin(), prow.end()), prow.end());
+  kp.nrows = (int)prow.size();
+  DKS_TRY(upload(&kp.plane_rows, prow.data(), prow.size()));
   DKS_TRY(upload(&kp.pw_stick, pstick.data(), pstick.size()));
   DKS_TRY(upload(&kp.pw_iz, piz.data(), piz.size()));
   DKS_TRY(upload(&kp.q, q.data(), q.size()));
   std::vector<float> cq(6 * (size_t)npw);
+  std::vector<double> cq64(3 * (size_t)npw);
   for (size_t e = 0; e < 3 * (size_t)npw; ++e) {
-    const double v = ctx->c * q[e];
+    const double v = cq64[e] = ctx->c * q[e];
     const float h = (float)v;
     cq[2 * e] = h;
     cq[2 * e + 1] = (float)(v - (double)h);
   }
   DKS_TRY(upload(&kp.cq32, cq.data(), cq.size()));
+  DKS_TRY(upload(&kp.cq64, cq64.data(), cq64.size()));
   DKS_TRY(upload(&kp.ek, ek.data(), ek.size()));
   // projector rows beta_c[(spin*npw + p)]
   if (!chans.empty()) {
@@ -273,8 +335,9 @@ static void free_ctx(dks_ctx* ctx) {
   if (!ctx) return;
   for (int a = 0; a < 3; ++a) {
     cudaFree(ctx->tw64[a]);
-    cudaFree(ctx->tw32[a]);
-    cudaFree(ctx->twdf[a]);
+    cudaFree(ctx->etw64[a]);
+    cudaFree(ctx->etw32[a]);
+    cudaFree(ctx->etwdf[a]);
   }
   cudaFree(ctx->vperm64);
   cudaFree(ctx->vperm32);
@@ -285,10 +348,12 @@ static void free_ctx(dks_ctx* ctx) {
   for (KPoint& kp : ctx->k) {
     cudaFree(kp.stick_start);
     cudaFree(kp.stick_plane);
+    cudaFree(kp.plane_rows);
     cudaFree(kp.pw_stick);
     cudaFree(kp.pw_iz);
     cudaFree(kp.q);
     cudaFree(kp.cq32);
+    cudaFree(kp.cq64);
     cudaFree(kp.ek);
     cudaFree(kp.bt64);
     cudaFree(kp.bt32);
@@ -379,22 +444,26 @@ int dks_create(const dks_cell* cell, double ecut, const dks_potentials* pot, con
   Bm[8] = tp * (a1[0] * a2[1] - a1[1] * a2[0]);
   // twiddles
   for (int a = 0; a < 3; ++a) {
-    const int n = ctx->grid[a];
-    std::vector<double2> tw(n);
-    std::vector<float2> tw32(n);
-    for (int t = 0; t < n; ++t) {
-      const double ang = 2.0 * 3.14159265358979323846 * t / n;
-      tw[t] = double2{std::cos(ang), std::sin(ang)};
-      tw32[t] = float2{(float)tw[t].x, (float)tw[t].y};
+    ctx->exec64[a] = make_exec_plan(ctx->plan[a], kExecRadix64);
+    ctx->exec32[a] = make_exec_plan(ctx->plan[a], kExecRadix32);
+    const std::vector<double2> tw = exec_twiddles(ctx->exec64[a]), t32 = exec_twiddles(ctx->exec32[a]);
+    std::vector<float2> tw32(t32.size());
+    for (size_t t = 0; t < t32.size(); ++t) tw32[t] = float2{(float)t32[t].x, (float)t32[t].y};
+    std::vector<float> twd;
+    for (const double2& w : tw)
+      for (double v : {w.x, w.y}) {
+        const float h = (float)v, l = (float)(v - (double)h);
+        twd.insert(twd.end(), {h, h, -h, -h, -l, -l});
+      }
+    std::vector<double2> nat(ctx->grid[a]);
+    for (int t = 0; t < ctx->grid[a]; ++t) {
+      const double ang = 2.0 * 3.14159265358979323846 * t / ctx->grid[a];
+      nat[t] = double2{std::cos(ang), std::sin(ang)};
     }
-    std::vector<float4> twd(n);
-    for (int t = 0; t < n; ++t) {
-      const float rh = (float)tw[t].x, ih = (float)tw[t].y;
-      twd[t] = float4{rh, (float)(tw[t].x - (double)rh), ih, (float)(tw[t].y - (double)ih)};
-    }
-    if ((rc = upload(&ctx->tw64[a], tw.data(), n))) return bail(rc);
-    if ((rc = upload(&ctx->tw32[a], tw32.data(), n))) return bail(rc);
-    if ((rc = upload(&ctx->twdf[a], twd.data(), n))) return bail(rc);
+    if ((rc = upload(&ctx->tw64[a], nat.data(), nat.size()))) return bail(rc);
+    if ((rc = upload(&ctx->etw64[a], tw.data(), tw.size()))) return bail(rc);
+    if ((rc = upload(&ctx->etw32[a], tw32.data(), tw32.size()))) return bail(rc);
+    if ((rc = upload(&ctx->etwdf[a], twd.data(), twd.size()))) return bail(rc);
   }
   // DIF positions of the natural grid indices (density and potential updates on the device)
   for (int a = 0; a < 3; ++a) {

@@ -46,6 +46,28 @@ bool make_axis_plan(int n, AxisPlan* p);
 // position of frequency index k after the DIF stages (mixed-radix digit reversal)
 std::vector<int> dif_positions(const AxisPlan& p);
 
+// What the kernels execute: the passes of an AxisPlan with neighbours merged (fft_device.cuh) up to
+// a largest radix, in DIF order, with the constants of their index arithmetic.  An axis of length 1
+// is one pass of radix 1.
+struct ExecPass {
+  int R;          // radix (merged: the product)
+  int S, L;       // block length L, sub-length S = L / R
+  unsigned mS;    // magic(S)
+  int tw;         // offset of its twiddles exp(2 pi i j r / L), [j < S][r < R], in the axis table (S > 1)
+};
+struct ExecPlan {
+  int n, nst;
+  int ntw;        // twiddles of the axis
+  int big;        // any merged radix
+  ExecPass p[kMaxStages];
+};
+ExecPlan make_exec_plan(const AxisPlan& a, int max_radix);
+constexpr int kTwDfFloats = 12;   // re: h h, -h -h, -l -l; im: the same
+constexpr int kExecRadix32 = 16, kExecRadix64 = 10;   // largest merged radix: 8-byte, 16-byte elements
+// ceil(2^32 / d): floor(a / d) = mulhi(a, magic(d)) for 0 <= a < 65536 and 1 < d < 65536; 0 stands
+// for d = 1
+inline unsigned magic(int d) { return d <= 1 ? 0u : (unsigned)(((1ull << 32) + (unsigned)d - 1) / (unsigned)d); }
+
 // --------------------------------------------------------------- per-k basis
 struct KPoint {
   int npw = 0;
@@ -57,9 +79,12 @@ struct KPoint {
   // device tables
   int* stick_start = nullptr;   // nsticks+1, pw offsets
   int* stick_plane = nullptr;   // nsticks, i1*LD + i2 (natural frequency position, padded rows)
+  int* plane_rows = nullptr;    // nrows, i1*LD of the rows of a plane that hold a stick
+  int nrows = 0;
   int* pw_stick = nullptr;      // npw
   int* pw_iz = nullptr;         // npw, i3 (natural)
   double* q = nullptr;          // npw*3 cartesian k+G (FP64)
+  double* cq64 = nullptr;       // npw*3, c (k+G)
   float* cq32 = nullptr;        // npw*6: c (k+G)_x, c (k+G)_y, c (k+G)_z as double-float (hi, lo) pairs
   double* ek = nullptr;         // npw, |k+G|^2/2
   double2* bt64 = nullptr;      // nproj x (2 npw) projector rows (beta, spin-major)
@@ -99,10 +124,13 @@ struct dks_ctx {
   int nk = 0;
   dks::AxisPlan plan[3];
   int plane_ld = 0;              // row stride of an N1 x N2 plane in shared memory (N2 rounded up to odd)
-  // device: twiddles exp(+2 pi i t / N_axis), t < N_axis
+  dks::ExecPlan exec32[3], exec64[3];   // executed passes for 8-byte and 16-byte elements
+  // device: twiddles of the executed passes (ExecPass::tw)
+  double2* etw64[3] = {nullptr, nullptr, nullptr};
+  float2* etw32[3] = {nullptr, nullptr, nullptr};
+  float* etwdf[3] = {nullptr, nullptr, nullptr};   // kTwDfFloats per twiddle (fft_device.cuh, ctw)
+  // device: exp(+2 pi i t / N_axis), t < N_axis (the direct transforms of the SCF grids)
   double2* tw64[3] = {nullptr, nullptr, nullptr};
-  float2* tw32[3] = {nullptr, nullptr, nullptr};
-  float4* twdf[3] = {nullptr, nullptr, nullptr};   // double-float twiddles (re hi, re lo, im hi, im lo)
   // device: V / Ng in DIF-permuted layout [p3][p1*LD + p2], zero in the padding column
   double* vperm64 = nullptr;
   float* vperm32 = nullptr;

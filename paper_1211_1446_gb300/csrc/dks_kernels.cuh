@@ -87,6 +87,20 @@ __device__ __forceinline__ dfl df_from_bits(double x) {
   const float lv = __uint2float_rn(lo32 & 0x1fffffffu) * __uint_as_float((unsigned)(e - 948) << 23);
   return dfl{h, sign ? -lv : lv};
 }
+// the same with h rounded to nearest (ties away from zero) instead of truncated, so that l keeps 24
+// of the remaining bits: h + l = x to 2^-49 relative.  (A conversion through the FP64 unit costs
+// four of its instructions, each worth some 75 FP32 ones on this part.)
+__device__ __forceinline__ dfl df_split_rn(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((unsigned)(u >> 52) & 0x7ffu);
+  if (e < 949 || e > 1149) return df_from(x);
+  const unsigned long long t = u + 0x10000000ull;            // a carry into the exponent is right
+  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+  const unsigned hb = (unsigned)((t & 0x7fffffffffffffffull) >> 29) - (896u << 23);
+  const int r = (int)((unsigned)t & 0x1fffffffu) - 0x10000000;   // |x| - |h| in units of 2^(e - 1075)
+  const float lv = __int2float_rn(r) * __uint_as_float((unsigned)(e - 948) << 23);
+  return dfl{__uint_as_float(hb | sign), __uint_as_float(__float_as_uint(lv) ^ sign)};
+}
 __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
   const float s = a.h + b.h;
   const float bb = s - a.h;
@@ -111,6 +125,32 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
   e = fmaf(a.l, b.h, e);
   const float h = p + e;
   return dfl{h, e - (h - p)};
+}
+
+// (h + l) 2^k as a double, from a normalised double-float pair (|l| <= ulp(h) / 2), with integer
+// operations only (FP64 instructions, conversions included, are slow on this part): the
+// significands are aligned in a 64-bit integer; exact up to a truncation below 2^-52 of h.
+// The caller keeps the result's exponent in range (|k| <= 60 and h a normal FP32 number).
+__device__ __forceinline__ double df_to_double(float h, float l, int k) {
+  const unsigned hb = __float_as_uint(h), lb = __float_as_uint(l);
+  const int eh = (int)((hb >> 23) & 255u);
+  if (eh == 0) return 0.0;
+  if (eh == 255) return __longlong_as_double(0x7FF8000000000000LL);   // NaN or infinity
+  long long m = (long long)((hb & 0x7FFFFFu) | 0x800000u) << 29;   // implicit bit at position 52
+  const int el = (int)((lb >> 23) & 255u);
+  if (el) {
+    const int d = eh - el;                                          // >= 24 for a normalised pair
+    if (d < 53) {
+      const long long ml = ((long long)((lb & 0x7FFFFFu) | 0x800000u) << 29) >> d;
+      m += ((hb ^ lb) >> 31) ? -ml : ml;
+    }
+  }
+  long long e = (long long)(eh - 127 + 1023 + k);
+  if (m < (1LL << 52)) {   // a borrow took the leading bit
+    m <<= 1;
+    --e;
+  }
+  return __longlong_as_double(((long long)(hb >> 31) << 63) | (e << 52) | (m & ((1LL << 52) - 1)));
 }
 
 // complex double-float (16 bytes, the size of a double2)

@@ -41,6 +41,7 @@
 #include <vector>
 
 #include "dks_internal.h"
+#include "dks_kernels.cuh"
 #include "tc_ptx.cuh"
 
 namespace dks {
@@ -191,32 +192,6 @@ __device__ __forceinline__ void df_add2(float& h, float& l, float h2, float l2) 
   l = e - (h - s);
 }
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }   // -126 <= k <= 127
-// (h + l) 2^k as a double, from a normalised double-float pair (|l| <= ulp(h) / 2), with integer
-// operations only (FP64 instructions, conversions included, are slow on this part): the
-// significands are aligned in a 64-bit integer; exact up to a truncation below 2^-52 of h.
-// The caller keeps the result's exponent in range (|k| <= 60 and h a normal FP32 number).
-__device__ __forceinline__ double df_to_double(float h, float l, int k) {
-  const uint32_t hb = __float_as_uint(h), lb = __float_as_uint(l);
-  const int eh = (int)((hb >> 23) & 255u);
-  if (eh == 0) return 0.0;
-  if (eh == 255) return __longlong_as_double(0x7FF8000000000000LL);   // NaN or infinity
-  long long m = (long long)((hb & 0x7FFFFFu) | 0x800000u) << 29;   // implicit bit at position 52
-  const int el = (int)((lb >> 23) & 255u);
-  if (el) {
-    const int d = eh - el;                                          // >= 24 for a normalised pair
-    if (d < 53) {
-      const long long ml = ((long long)((lb & 0x7FFFFFu) | 0x800000u) << 29) >> d;
-      m += ((hb ^ lb) >> 31) ? -ml : ml;
-    }
-  }
-  long long e = (long long)(eh - 127 + 1023 + k);
-  if (m < (1LL << 52)) {   // a borrow took the leading bit
-    m <<= 1;
-    --e;
-  }
-  return __longlong_as_double(((long long)(hb >> 31) << 63) | (e << 52) | (m & ((1LL << 52) - 1)));
-}
-
 // ================================================================ Gram: A = Z^H HZ, S = Z^H Z
 // A tile is 128 columns of Z (MMA M) against 48 columns of HZ (A) or of Z (S), over a chunk of
 // whole windows.  Warp 0: TMA producer (per 16-row stage one 5-D copy of the A slices and one
