@@ -244,7 +244,7 @@ static int build_k(dks_ctx* ctx, const double kfrac[3], double ecut, const dks_p
         return fail(DKS_ERR_GRID, "planewave sphere does not fit the FFT grid along axis " + std::to_string(a));
   kp.npw = npw;
   kp.miller = mil;
-  std::vector<int> sstart, splane, pstick(npw), piz(npw);
+  std::vector<int> sstart, splane, sfirst, pat(npw);
   std::vector<double> ek(npw);
   double qmax2 = 0;
   for (int p = 0; p < npw; ++p) {
@@ -254,8 +254,9 @@ static int build_k(dks_ctx* ctx, const double kfrac[3], double ecut, const dks_p
       const int i2 = ((mil[3 * p + 1] % ctx->grid[1]) + ctx->grid[1]) % ctx->grid[1];
       splane.push_back(i1 * ctx->plane_ld + i2);
     }
-    pstick[p] = (int)sstart.size() - 1;
-    piz[p] = ((mil[3 * p + 2] % ctx->grid[2]) + ctx->grid[2]) % ctx->grid[2];
+    const int i3 = ((mil[3 * p + 2] % ctx->grid[2]) + ctx->grid[2]) % ctx->grid[2];
+    if (sfirst.size() < sstart.size()) sfirst.push_back(i3);
+    pat[p] = ((int)sstart.size() - 1) * 256 + i3;   // i3 < 256, fewer than 2^16 sticks
     const double q2 = q[3 * p] * q[3 * p] + q[3 * p + 1] * q[3 * p + 1] + q[3 * p + 2] * q[3 * p + 2];
     ek[p] = 0.5 * q2;
     qmax2 = std::max(qmax2, q2);
@@ -271,8 +272,8 @@ static int build_k(dks_ctx* ctx, const double kfrac[3], double ecut, const dks_p
   prow.erase(std::unique(prow.begin(), prow.end()), prow.end());
   kp.nrows = (int)prow.size();
   DKS_TRY(upload(&kp.plane_rows, prow.data(), prow.size()));
-  DKS_TRY(upload(&kp.pw_stick, pstick.data(), pstick.size()));
-  DKS_TRY(upload(&kp.pw_iz, piz.data(), piz.size()));
+  DKS_TRY(upload(&kp.stick_first, sfirst.data(), sfirst.size()));
+  DKS_TRY(upload(&kp.pw_at, pat.data(), pat.size()));
   DKS_TRY(upload(&kp.q, q.data(), q.size()));
   std::vector<float> cq(6 * (size_t)npw);
   std::vector<double> cq64(3 * (size_t)npw);
@@ -349,8 +350,8 @@ static void free_ctx(dks_ctx* ctx) {
     cudaFree(kp.stick_start);
     cudaFree(kp.stick_plane);
     cudaFree(kp.plane_rows);
-    cudaFree(kp.pw_stick);
-    cudaFree(kp.pw_iz);
+    cudaFree(kp.stick_first);
+    cudaFree(kp.pw_at);
     cudaFree(kp.q);
     cudaFree(kp.cq32);
     cudaFree(kp.cq64);

@@ -81,8 +81,8 @@ struct KPoint {
   int* stick_plane = nullptr;   // nsticks, i1*LD + i2 (natural frequency position, padded rows)
   int* plane_rows = nullptr;    // nrows, i1*LD of the rows of a plane that hold a stick
   int nrows = 0;
-  int* pw_stick = nullptr;      // npw
-  int* pw_iz = nullptr;         // npw, i3 (natural)
+  int* stick_first = nullptr;   // nsticks, i3 of the stick's first planewave
+  int* pw_at = nullptr;         // npw, stick * 256 + i3 (natural)
   double* q = nullptr;          // npw*3 cartesian k+G (FP64)
   double* cq64 = nullptr;       // npw*3, c (k+G)
   float* cq32 = nullptr;        // npw*6: c (k+G)_x, c (k+G)_y, c (k+G)_z as double-float (hi, lo) pairs

@@ -87,13 +87,16 @@ __device__ __forceinline__ dfl df_from_bits(double x) {
   const float lv = __uint2float_rn(lo32 & 0x1fffffffu) * __uint_as_float((unsigned)(e - 948) << 23);
   return dfl{h, sign ? -lv : lv};
 }
+// out of line, so that the FP64 instructions are not if-converted into the callers' main path (a
+// predicated-off FP64 instruction still takes its slot of that unit)
+static __device__ __noinline__ dfl df_from_call(double x) { return df_from(x); }
 // the same with h rounded to nearest (ties away from zero) instead of truncated, so that l keeps 24
 // of the remaining bits: h + l = x to 2^-49 relative.  (A conversion through the FP64 unit costs
 // four of its instructions, each worth some 75 FP32 ones on this part.)
 __device__ __forceinline__ dfl df_split_rn(double x) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((unsigned)(u >> 52) & 0x7ffu);
-  if (e < 949 || e > 1149) return df_from(x);
+  if (e < 949 || e > 1149) return df_from_call(x);
   const unsigned long long t = u + 0x10000000ull;            // a carry into the exponent is right
   const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
   const unsigned hb = (unsigned)((t & 0x7fffffffffffffffull) >> 29) - (896u << 23);

@@ -297,12 +297,25 @@ __device__ __forceinline__ void dft_pq(const V* x, V* y) {
 // a / d for 0 <= a < 65536 by m = magic(d) = ceil(2^32 / d) (0 stands for d = 1)
 __device__ __forceinline__ int mdiv(int a, unsigned m) { return m ? (int)__umulhi((unsigned)a, m) : a; }
 
-// the nlines lines a pass runs over: line l starts at rows[l] (a table in shared memory) or at
-// l * lstride; its element i is es elements further per unit.  mN = magic(nlines)
+// the n lines a pass runs over: line l starts at rows[l] (a table in shared memory) or at l * lstride;
+// its element i is es elements further per unit.  mN = magic(n)
 struct Lines {
   const int* rows;
   int lstride, es, n;
   unsigned mN;
+};
+
+// Where a pass reads and writes: shared memory in place; or the last DIF pass storing straight to
+// the stick buffer T; or the first DIT pass loading straight from it (T[component][position][stick],
+// consecutive lines of a component are consecutive sticks, so both are coalesced).  The stick
+// kernels save a trip through shared memory, a barrier and a loop that way.
+enum PassIO { kInPlace, kStoreT, kLoadT };
+template <typename V>
+struct StickBuf {
+  V* t;             // T at the CTA's first stick
+  int nsticks, ns;  // stick count (the stride of a position), sticks of this CTA
+  int lspb;         // log2 of the lines per component in shared memory
+  size_t comp;      // stride of a component
 };
 
 // one execution pass of radix R = P Q (P then Q of the axis plan; Q = 1: a plain radix).
@@ -311,10 +324,10 @@ struct Lines {
 //   vmid (only where S = 1): the last DIF pass of an inverse transform, the product with the real
 //   factors vmid[offset] and the first DIT pass of the forward transform in one, without a trip
 //   through shared memory between them; the result is swapped data
-template <typename V, int P, int Q>
+template <typename V, int P, int Q, PassIO IO>
 __device__ __forceinline__ void fft_pass(V* __restrict__ buf, const Lines& ln, const ExecPass& p, int n,
                                          const typename TwOf<V>::T* __restrict__ tw, bool dit,
-                                         const typename RealOf<V>::T* __restrict__ vmid) {
+                                         const typename RealOf<V>::T* __restrict__ vmid, const StickBuf<V>& sb) {
   constexpr int R = P * Q;
   const int S = p.S;
   const int total = ln.n * (n / R);
@@ -325,16 +338,22 @@ __device__ __forceinline__ void fft_pass(V* __restrict__ buf, const Lines& ln, c
     const int line = t - u * ln.n;
     const int blk = mdiv(u, p.mS);
     const int j = u - blk * S;
-    V* base = buf + (ln.rows ? ln.rows[line] : line * ln.lstride) + (blk * p.L + j) * ln.es;
-    V x[R], y[R];
-    if (Q > 1 && dit) {
-      sfor<0, R>([&](auto rc) {
-        constexpr int r = decltype(rc)::value;
-        x[r] = base[((r % P) * Q + r / P) * se];
-      });
-    } else {
-      sfor<0, R>([&](auto rc) { x[decltype(rc)::value] = base[decltype(rc)::value * se]; });
+    const int pos = blk * p.L + j;
+    V* base = buf + (ln.rows ? ln.rows[line] : line * ln.lstride) + pos * ln.es;
+    V* gbase = nullptr;
+    if constexpr (IO != kInPlace) {
+      const int s = line & ((1 << sb.lspb) - 1);
+      if (s >= sb.ns) continue;   // beyond the last stick
+      gbase = sb.t + (size_t)(line >> sb.lspb) * sb.comp + (size_t)pos * sb.nsticks + s;
     }
+    const int gse = S * sb.nsticks;
+    V x[R], y[R];
+    sfor<0, R>([&](auto rc) {
+      constexpr int r = decltype(rc)::value, sr = (r % P) * Q + r / P;
+      const int slot = Q > 1 && dit ? sr : r;
+      if constexpr (IO == kLoadT) x[r] = gbase[(size_t)slot * gse];
+      else x[r] = base[slot * se];
+    });
     if (dit && j) {
       const typename TwOf<V>::T* w = tw + j * R;
       sfor<1, R>([&](auto rc) { x[decltype(rc)::value] = cmul(x[decltype(rc)::value], w[decltype(rc)::value]); });
@@ -359,42 +378,41 @@ __device__ __forceinline__ void fft_pass(V* __restrict__ buf, const Lines& ln, c
       const typename TwOf<V>::T* w = tw + j * R;
       sfor<1, R>([&](auto rc) { y[decltype(rc)::value] = cmul(y[decltype(rc)::value], w[decltype(rc)::value]); });
     }
-    if (Q > 1 && !dit && !vmid) {
-      sfor<0, R>([&](auto rc) {
-        constexpr int r = decltype(rc)::value;
-        base[((r % P) * Q + r / P) * se] = y[r];
-      });
-    } else {
-      sfor<0, R>([&](auto rc) { base[decltype(rc)::value * se] = y[decltype(rc)::value]; });
-    }
+    sfor<0, R>([&](auto rc) {
+      constexpr int r = decltype(rc)::value, sr = (r % P) * Q + r / P;
+      const int slot = Q > 1 && !dit && !vmid ? sr : r;
+      if constexpr (IO == kStoreT) gbase[(size_t)slot * gse] = y[r];
+      else base[slot * se] = y[r];
+    });
   }
 }
 
 // one pass of any radix, and the barrier after it.  BIG: plans with merged radices (more registers)
-template <typename V, bool BIG>
+template <typename V, bool BIG, PassIO IO = kInPlace>
 __device__ __forceinline__ void fft_step(V* buf, const Lines& ln, const ExecPass& p, int n,
-                                         const typename TwOf<V>::T* tw, bool dit, const typename RealOf<V>::T* vmid) {
+                                         const typename TwOf<V>::T* tw, bool dit, const typename RealOf<V>::T* vmid,
+                                         const StickBuf<V>& sb = {}) {
   switch (p.R) {
-    case 1: fft_pass<V, 1, 1>(buf, ln, p, n, tw, dit, vmid); break;
-    case 2: fft_pass<V, 2, 1>(buf, ln, p, n, tw, dit, vmid); break;
-    case 3: fft_pass<V, 3, 1>(buf, ln, p, n, tw, dit, vmid); break;
-    case 4: fft_pass<V, 4, 1>(buf, ln, p, n, tw, dit, vmid); break;
-    case 5: fft_pass<V, 5, 1>(buf, ln, p, n, tw, dit, vmid); break;
-    case 6: fft_pass<V, 6, 1>(buf, ln, p, n, tw, dit, vmid); break;
-    case 7: fft_pass<V, 7, 1>(buf, ln, p, n, tw, dit, vmid); break;
-    case 8: fft_pass<V, 8, 1>(buf, ln, p, n, tw, dit, vmid); break;
+    case 1: fft_pass<V, 1, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+    case 2: fft_pass<V, 2, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+    case 3: fft_pass<V, 3, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+    case 4: fft_pass<V, 4, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+    case 5: fft_pass<V, 5, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+    case 6: fft_pass<V, 6, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+    case 7: fft_pass<V, 7, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+    case 8: fft_pass<V, 8, 1, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
     default:
       if constexpr (BIG) {
         switch (p.R) {
-          case 9: fft_pass<V, 3, 3>(buf, ln, p, n, tw, dit, vmid); break;
-          case 10: fft_pass<V, 5, 2>(buf, ln, p, n, tw, dit, vmid); break;
+          case 9: fft_pass<V, 3, 3, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+          case 10: fft_pass<V, 5, 2, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
           default:
             if constexpr (sizeof(V) == sizeof(float2)) {
               switch (p.R) {
-                case 12: fft_pass<V, 6, 2>(buf, ln, p, n, tw, dit, vmid); break;
-                case 14: fft_pass<V, 7, 2>(buf, ln, p, n, tw, dit, vmid); break;
-                case 15: fft_pass<V, 5, 3>(buf, ln, p, n, tw, dit, vmid); break;
-                default: fft_pass<V, 8, 2>(buf, ln, p, n, tw, dit, vmid); break;
+                case 12: fft_pass<V, 6, 2, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+                case 14: fft_pass<V, 7, 2, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+                case 15: fft_pass<V, 5, 3, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
+                default: fft_pass<V, 8, 2, IO>(buf, ln, p, n, tw, dit, vmid, sb); break;
               }
             }
         }
@@ -414,10 +432,44 @@ __device__ __forceinline__ void fft_axis(V* buf, const Lines& ln, const ExecPlan
   }
 }
 
+// the inverse transform of the lines of axis 3 in shared memory, its last pass storing to T, and the
+// forward transform from T, its first pass loading from there
+template <typename V, bool BIG>
+__device__ __forceinline__ void fft_axis_store(V* buf, const Lines& ln, const ExecPlan& e,
+                                               const typename TwOf<V>::T* tw, const StickBuf<V>& sb) {
+#pragma unroll 1
+  for (int i = 0; i + 1 < e.nst; ++i) fft_step<V, BIG>(buf, ln, e.p[i], e.n, tw + e.p[i].tw, false, nullptr);
+  const ExecPass& p = e.p[e.nst - 1];
+  fft_step<V, BIG, kStoreT>(buf, ln, p, e.n, tw + p.tw, false, nullptr, sb);
+}
+template <typename V, bool BIG>
+__device__ __forceinline__ void fft_axis_load(V* buf, const Lines& ln, const ExecPlan& e,
+                                              const typename TwOf<V>::T* tw, const StickBuf<V>& sb) {
+  const ExecPass& p = e.p[e.nst - 1];
+  fft_step<V, BIG, kLoadT>(buf, ln, p, e.n, tw + p.tw, true, nullptr, sb);
+#pragma unroll 1
+  for (int i = e.nst - 2; i >= 0; --i) fft_step<V, BIG>(buf, ln, e.p[i], e.n, tw + e.p[i].tw, true, nullptr);
+}
+
 // copies n twiddles into shared memory (the caller's next barrier publishes them)
 template <typename TW>
 __device__ __forceinline__ void load_twiddles(TW* dst, const TW* __restrict__ src, int n) {
   for (int e = threadIdx.x; e < n; e += blockDim.x) dst[e] = src[e];
 }
 
+// shared memory of n twiddles, with room for their alignment
+template <typename V>
+static size_t twiddle_bytes(int n) {
+  return n * sizeof(typename TwOf<V>::T) + 16;
+}
+
+// Pass B in one kernel needs the whole N1 x LD plane in shared memory; larger planes (or a
+// tuner's choice, ctx->plane_split) take the three-kernel form through the buffer P.
+template <typename V>
+static bool split_plane(const dks_ctx* ctx) {
+  const ExecPlan* e = sizeof(V) == sizeof(float2) ? ctx->exec32 : ctx->exec64;
+  const size_t need = (size_t)ctx->grid[0] * ctx->plane_ld * sizeof(V) + twiddle_bytes<V>(e[0].ntw + e[1].ntw) +
+                      ctx->grid[0] * sizeof(int);
+  return ctx->plane_split || need > 227 * 1024;
+}
 }  // namespace dks
