@@ -2,9 +2,8 @@
 //
 //  gemm_hn   C (m x n) += A^H B   A: k x m, B: k x n (k = 4 npw or 2 npw, huge; m, n small)
 //            Gram matrices of the projected pencil and the projector coefficients B^H x~.
-//            Split over k across the grid; each CTA reduces a 32x32 tile of C over its
-//            k-range in registers and adds it to C with FP64 atomics.  With FP32 operands
-//            each 32-deep k-tile is summed in FP32 and folded into a double-float total.
+//            Split over k across the grid; each CTA reduces a tile of C over its k-range in
+//            registers and adds it to C with FP64 atomics.
 //  gemm_nn   OUT (k x n) = alpha A (k x m) diag(ws) W (m x n) + beta OUT
 //            Rotations X <- Z V, P <- [0,Y,P] V and the projector
 //            update x~ += B (D Z).  W (FP64, from the small solve) is staged in shared
@@ -46,18 +45,25 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
-// RM = 2: 32 x 32 tiles of C; RM = 3: 48 x 32 tiles (less padding when m is just above 32)
-template <typename Va, typename Vb, typename A, int RM>
-__global__ void __launch_bounds__(256) k_gemm_hn(const Va* __restrict__ a, int lda, const Vb* __restrict__ b,
-                                                 int ldb, int k, int m, int n, int mt, int kchunk,
-                                                 double2* __restrict__ c, int ldc, int lower) {
-  constexpr int TM = 16 * RM;
-  __shared__ A as[HN_T][TM + 1];
-  __shared__ A bs[HN_T][HN_T + 1];
+// FP64 arithmetic (either operand complex128, or Acc64).  Bound by the FP64 unit: 1.7 fused
+// multiply-adds per clock and SM, so a warp's multiply-add takes 19 cycles of the whole SM and a
+// shared-memory operand per complex multiply-add is free beside it.  What counts is that every SM
+// has work and that none of it is padding: one output per thread, 16 x 16 tiles, and the k range
+// split until there are about four CTAs per SM.  (36 projector channels, 18 columns, 574 rows: 56 us
+// with 48 x 32 tiles, whose 18 CTAs multiplied 2.4 x the outputs.)
+constexpr int HD_T = 16, HD_K = 32;
+
+template <typename Va, typename Vb>
+__global__ void __launch_bounds__(HD_T * HD_T) k_gemm_hn64(const Va* __restrict__ a, int lda,
+                                                           const Vb* __restrict__ b, int ldb, int k, int m, int n,
+                                                           int mt, int kchunk, double2* __restrict__ c, int ldc,
+                                                           int lower) {
+  __shared__ double2 as[HD_K][HD_T + 1];
+  __shared__ double2 bs[HD_K][HD_T + 1];
   int tm, tn;
   if (lower) {   // only tiles with tn <= tm (the block lower triangle of a Hermitian result)
     const int t = blockIdx.x;
-    tm = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+    tm = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
     while ((tm + 1) * (tm + 2) / 2 <= t) ++tm;
     while (tm * (tm + 1) / 2 > t) --tm;
     tn = t - tm * (tm + 1) / 2;
@@ -65,72 +71,44 @@ __global__ void __launch_bounds__(256) k_gemm_hn(const Va* __restrict__ a, int l
     tm = blockIdx.x % mt;
     tn = blockIdx.x / mt;
   }
-  const int m0 = tm * TM, n0 = tn * HN_T;
+  const int m0 = tm * HD_T, n0 = tn * HD_T;
   const int kb = blockIdx.y * kchunk;
   const int ke = min(k, kb + kchunk);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  A acc[RM][2];
-#pragma unroll
-  for (int i = 0; i < RM; ++i) acc[i][0] = acc[i][1] = A{0, 0};
-  // FP32 arithmetic: each k-tile is summed in FP32 and folded into a double-float total, so
-  // FP32 rounding accumulates over 32 terms instead of the whole k-range of the CTA
-  constexpr bool fold = std::is_same<A, float2>::value;
-  dfl tot[RM][2][2] = {};
-  for (int k0 = kb; k0 < ke; k0 += HN_T) {
-    for (int e = threadIdx.x; e < HN_T * TM; e += 256) {
-      const int kq = e & (HN_T - 1), q = e >> 5;
+  // a warp holds 8 x 4 outputs; warps whose outputs all lie outside C only help loading
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int ty = (w & 1) * 8 + (lane & 7), tx = (w >> 1) * 4 + (lane >> 3);
+  const bool live = m0 + (w & 1) * 8 < m && n0 + (w >> 1) * 4 < n;
+  double2 acc{0, 0};
+  for (int k0 = kb; k0 < ke; k0 += HD_K) {
+    for (int e = threadIdx.x; e < HD_K * HD_T; e += HD_T * HD_T) {
+      const int kq = e & (HD_K - 1), q = e >> 5;
       const int gk = k0 + kq;
-      A va{0, 0};
-      if (gk < ke && m0 + q < m) va = cvt<A>(a[(size_t)(m0 + q) * lda + gk]);
+      double2 va{0, 0}, vb{0, 0};
+      if (gk < ke && m0 + q < m) va = cvt<double2>(a[(size_t)(m0 + q) * lda + gk]);
+      if (gk < ke && n0 + q < n) vb = cvt<double2>(b[(size_t)(n0 + q) * ldb + gk]);
       as[kq][q] = va;
-    }
-    for (int e = threadIdx.x; e < HN_T * HN_T; e += 256) {
-      const int kq = e & (HN_T - 1), q = e >> 5;
-      const int gk = k0 + kq;
-      A vb{0, 0};
-      if (gk < ke && n0 + q < n) vb = cvt<A>(b[(size_t)(n0 + q) * ldb + gk]);
       bs[kq][q] = vb;
     }
     __syncthreads();
-#pragma unroll 8
-    for (int kq = 0; kq < HN_T; ++kq) {
-      const A b0 = bs[kq][tx], b1 = bs[kq][tx + 16];
-#pragma unroll
-      for (int i = 0; i < RM; ++i) {
-        const A ai = as[kq][ty + 16 * i];
-        acc[i][0] = cfmac(ai, b0, acc[i][0]);
-        acc[i][1] = cfmac(ai, b1, acc[i][1]);
-      }
-    }
-    if constexpr (fold) {
-#pragma unroll
-      for (int i = 0; i < RM; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          tot[i][j][0] = df_add_f(tot[i][j][0], acc[i][j].x);
-          tot[i][j][1] = df_add_f(tot[i][j][1], acc[i][j].y);
-          acc[i][j] = A{0, 0};
-        }
+    if (live) {
+      const int kn = min(HD_K, ke - k0);
+#pragma unroll 4
+      for (int kq = 0; kq < kn; ++kq) acc = cfmac(as[kq][ty], bs[kq][tx], acc);
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < RM; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int mm = m0 + ty + 16 * i, nn = n0 + tx + 16 * j;
-      if (mm < m && nn < n) {
-        const double vx = fold ? df_val(tot[i][j][0]) : (double)acc[i][j].x;
-        const double vy = fold ? df_val(tot[i][j][1]) : (double)acc[i][j].y;
-        atomicAdd(&c[(size_t)nn * ldc + mm].x, vx);
-        atomicAdd(&c[(size_t)nn * ldc + mm].y, vy);
-      }
-    }
+  const int mm = m0 + ty, nn = n0 + tx;
+  if (mm < m && nn < n) {
+    atomicAdd(&c[(size_t)nn * ldc + mm].x, acc.x);
+    atomicAdd(&c[(size_t)nn * ldc + mm].y, acc.y);
+  }
 }
 
-// The FP32 case of k_gemm_hn (complex64 operands, FP32 k-tiles folded into double-float totals)
-// with two shared-memory stages: the next 32-deep k-tile of A and B is copied with cp.async
-// while the current one is multiplied.
+// FP32 arithmetic (complex64 operands): each 32-deep k-tile is summed in FP32 and folded into a
+// double-float total, so FP32 rounding accumulates over 32 terms instead of the whole k-range of
+// the CTA; two shared-memory stages: the next k-tile of A and B is copied with cp.async while the
+// current one is multiplied.  RM = 2: 32 x 32 tiles of C; RM = 3: 48 x 32 tiles (less padding when m
+// is just above 32).
 template <int RM>
 constexpr size_t hn32_smem() {
   return 2 * ((size_t)HN_T * (16 * RM + 1) + (size_t)HN_T * (HN_T + 1)) * sizeof(float2);
@@ -368,12 +346,15 @@ int gemm_hn(const Va* a, int lda, const Vb* b, int ldb, int k, int m, int n, dou
       return tc_gemm_hn(a, lda, b, ldb, k, m, n, c, ldc, false, st, num_sms());
     }
   }
-  // 48-row tiles when they pad m less than 32-row tiles (not for the square lower-triangle mode)
-  const bool rm3 = !lower && (m + 47) / 48 * 48 < (m + 31) / 32 * 32;
-  const int tmr = rm3 ? 48 : HN_T;
-  const int mt = (m + tmr - 1) / tmr, nt = (n + HN_T - 1) / HN_T;
+  using A = typename std::conditional<Acc64, double2, typename AccOf<Va, Vb>::T>::type;
+  constexpr bool acc32 = std::is_same<A, float2>::value;
+  // FP32: 48-row tiles when they pad m less than 32-row tiles (not for the square lower-triangle mode)
+  const bool rm3 = acc32 && !lower && (m + 47) / 48 * 48 < (m + 31) / 32 * 32;
+  const int tmr = acc32 ? (rm3 ? 48 : HN_T) : HD_T, tnr = acc32 ? HN_T : HD_T;
+  const int mt = (m + tmr - 1) / tmr, nt = (n + tnr - 1) / tnr;
   const int tiles = lower ? mt * (mt + 1) / 2 : mt * nt;
   const int ktiles = (k + HN_T - 1) / HN_T;
+  static_assert(HD_K == HN_T, "one k-tile length");
   int splits = std::max(1, (4 * num_sms()) / tiles);
   splits = std::min(splits, ktiles);
   const int kchunk = ((ktiles + splits - 1) / splits) * HN_T;
@@ -384,9 +365,7 @@ int gemm_hn(const Va* a, int lda, const Vb* b, int ldb, int k, int m, int n, dou
   Prof pr(f32 && cat < P_RR ? cat + kProf32 : cat, st, (same ? (double)m * sizeof(Va) : (double)m * sizeof(Va) + (double)n * sizeof(Vb)) * k +
                        16.0 * m * n,
           (lower ? 4.0 * m * (m + 1.0) : 8.0 * m * n) * (double)k);
-  using A = typename std::conditional<Acc64, double2, typename AccOf<Va, Vb>::T>::type;
-  if constexpr (std::is_same<A, float2>::value && std::is_same<Va, float2>::value &&
-                std::is_same<Vb, float2>::value) {
+  if constexpr (acc32) {
     static bool attr = false;
     if (!attr) {
       DKS_CUDA_TRY(cudaFuncSetAttribute((const void*)k_gemm_hn_f32p<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -399,10 +378,8 @@ int gemm_hn(const Va* a, int lda, const Vb* b, int ldb, int k, int m, int n, dou
       k_gemm_hn_f32p<3><<<grid, 256, hn32_smem<3>(), st>>>(a, lda, b, ldb, k, m, n, mt, kchunk, c, ldc, lower ? 1 : 0);
     else
       k_gemm_hn_f32p<2><<<grid, 256, hn32_smem<2>(), st>>>(a, lda, b, ldb, k, m, n, mt, kchunk, c, ldc, lower ? 1 : 0);
-  } else if (rm3) {
-    k_gemm_hn<Va, Vb, A, 3><<<grid, 256, 0, st>>>(a, lda, b, ldb, k, m, n, mt, kchunk, c, ldc, lower ? 1 : 0);
   } else {
-    k_gemm_hn<Va, Vb, A, 2><<<grid, 256, 0, st>>>(a, lda, b, ldb, k, m, n, mt, kchunk, c, ldc, lower ? 1 : 0);
+    k_gemm_hn64<Va, Vb><<<grid, HD_T * HD_T, 0, st>>>(a, lda, b, ldb, k, m, n, mt, kchunk, c, ldc, lower ? 1 : 0);
   }
   DKS_CUDA_TRY(cudaGetLastError());
   return DKS_OK;
@@ -468,63 +445,63 @@ int mirror_lower(double2* c, int m, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------- gemm_nn
-constexpr int NN_R = 64, NN_C = 32, NN_M = 16;
+// FP64 arithmetic.  As in k_gemm_hn64 the FP64 unit is all that counts: a warp takes 32 rows and NC
+// columns of OUT, with the W columns of the CTA in shared memory (broadcast reads) and A read through
+// L1 (one 512-byte load per NC complex multiply-adds, of 76 SM cycles each).  No output and no inner
+// index is padding; NC is the largest that still gives every SM eight warps.  (36 inner indices, 18
+// columns, 574 rows: 108 us with 64 x 32 tiles, which left 9 CTAs with 2.4 x the multiply-adds.)
+constexpr int ND_WARPS = 4;
+constexpr int ND_M = 64;   // inner indices staged at a time
 
-template <typename Va, typename Vo>
-__global__ void __launch_bounds__(256) k_gemm_nn(const Va* __restrict__ a, int lda, int k, int m,
-                                                 const double2* __restrict__ w, int ldw,
-                                                 const double* __restrict__ ws, int n, Vo* __restrict__ out,
-                                                 int ldo, double alpha, double beta) {
-  using A = typename AccOf<Va, Vo>::T;
-  __shared__ A as[NN_M][NN_R];
-  __shared__ A wsm[NN_M][NN_C];
-  const int r0 = blockIdx.x * NN_R, c0 = blockIdx.y * NN_C;
-  const int row = threadIdx.x & (NN_R - 1), cg = threadIdx.x >> 6;
-  A acc[8];
+template <typename Va, typename Vo, int NC>
+__global__ void __launch_bounds__(32 * ND_WARPS) k_gemm_nn64(const Va* __restrict__ a, int lda, int k, int m,
+                                                             const double2* __restrict__ w, int ldw,
+                                                             const double* __restrict__ ws, int n,
+                                                             Vo* __restrict__ out, int ldo, double alpha, double beta) {
+  __shared__ double2 wsm[ND_WARPS * NC][ND_M];
+  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+  const int row = blockIdx.x * 32 + lane, cb = blockIdx.y * (ND_WARPS * NC), c0 = cb + wl * NC;
+  const int nc = min(NC, n - c0);      // columns of this warp (none: it only helps staging W)
+  double2 acc[NC];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) acc[j] = A{0, 0};
-  for (int m0 = 0; m0 < m; m0 += NN_M) {
-    for (int e = threadIdx.x; e < NN_M * NN_R; e += 256) {
-      const int rr = e & (NN_R - 1), mm = e >> 6;
-      A v{0, 0};
-      if (m0 + mm < m && r0 + rr < k) v = cvt<A>(a[(size_t)(m0 + mm) * lda + r0 + rr]);
-      as[mm][rr] = v;
-    }
-    for (int e = threadIdx.x; e < NN_M * NN_C; e += 256) {
-      const int cc = e & (NN_C - 1), mm = e >> 5;
+  for (int j = 0; j < NC; ++j) acc[j] = double2{0, 0};
+  for (int m0 = 0; m0 < m; m0 += ND_M) {
+    const int mn = min(ND_M, m - m0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < ND_WARPS * NC * ND_M; e += 32 * ND_WARPS) {
+      const int mm = e & (ND_M - 1), cc = e / ND_M;
       double2 v{0, 0};
-      if (m0 + mm < m && c0 + cc < n) {
-        v = w[(size_t)(c0 + cc) * ldw + m0 + mm];
+      if (mm < mn && cb + cc < n) {
+        v = w[(size_t)(cb + cc) * ldw + m0 + mm];
         const double s = (ws ? ws[m0 + mm] : 1.0) * alpha;
         v.x *= s;
         v.y *= s;
       }
-      wsm[mm][cc] = cvt<A>(v);
+      wsm[cc][mm] = v;
     }
     __syncthreads();
+    if (nc <= 0 || row >= k) continue;
+    const Va* ap = a + (size_t)m0 * lda + row;
 #pragma unroll 4
-    for (int mm = 0; mm < NN_M; ++mm) {
-      const A av = as[mm][row];
+    for (int mm = 0; mm < mn; ++mm) {
+      const double2 av = cvt<double2>(ap[(size_t)mm * lda]);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = cfma(av, wsm[mm][cg * 8 + j], acc[j]);
+      for (int j = 0; j < NC; ++j)
+        if (j < nc) acc[j] = cfma(av, wsm[wl * NC + j][mm], acc[j]);
     }
-    __syncthreads();
   }
-  if (r0 + row < k) {
+  if (row >= k) return;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int cc = c0 + cg * 8 + j;
-      if (cc < n) {
-        Vo* o = out + (size_t)cc * ldo + r0 + row;
-        A r = acc[j];
-        if (beta != 0.0) {
-          const A old = cvt<A>(*o);
-          r.x += (typename RealOf<A>::T)beta * old.x;
-          r.y += (typename RealOf<A>::T)beta * old.y;
-        }
-        *o = from_d2<Vo>(to_d2(r));
-      }
+  for (int j = 0; j < NC; ++j) {
+    if (j >= nc) break;
+    Vo* o = out + (size_t)(c0 + j) * ldo + row;
+    double2 r = acc[j];
+    if (beta != 0.0) {
+      const double2 old = cvt<double2>(*o);
+      r.x += beta * old.x;
+      r.y += beta * old.y;
     }
+    *o = from_d2<Vo>(r);
   }
 }
 
@@ -679,8 +656,15 @@ int gemm_nn(const Va* a, int lda, int k, int m, const double2* w, int ldw, const
     }
     k_gemm_nn_f32<<<grid, 64 * g, NF_SMEM, st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, (float)beta);
   } else {
-    dim3 grid((k + NN_R - 1) / NN_R, (n + NN_C - 1) / NN_C);
-    k_gemm_nn<Va, Vo><<<grid, 256, 0, st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, beta);
+    const int rb = (k + 31) / 32;
+    const long long warps = (long long)rb * n;
+    auto grid = [&](int nc) { return dim3(rb, (n + ND_WARPS * nc - 1) / (ND_WARPS * nc)); };
+    if (warps >= 32LL * num_sms() && n > 2 * ND_WARPS)
+      k_gemm_nn64<Va, Vo, 4><<<grid(4), 32 * ND_WARPS, 0, st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, beta);
+    else if (warps >= 16LL * num_sms() && n > ND_WARPS)
+      k_gemm_nn64<Va, Vo, 2><<<grid(2), 32 * ND_WARPS, 0, st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, beta);
+    else
+      k_gemm_nn64<Va, Vo, 1><<<grid(1), 32 * ND_WARPS, 0, st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, beta);
   }
   DKS_CUDA_TRY(cudaGetLastError());
   return DKS_OK;
