@@ -12,7 +12,7 @@
 //     chol_tol the kernel records it and returns -- the single-CTA kernel then runs
 //     the SVQB path
 //  3. W = L^-1 A' and C = L^-1 W^H = L^-1 A' L^-H: column-oriented forward substitution,
-//     warp per right-hand side, no reductions
+//     CTA per right-hand side, no reductions
 //  4. Householder reduction of C to a complex tridiagonal with the columns of C distributed
 //     over the shared memories of the cluster (column j in CTA j % csize); reflectors and
 //     p = tau C v travel through distributed shared memory; two barriers per column
@@ -22,7 +22,12 @@
 //  6. eigenvectors by inverse iteration on the tridiagonal (LU with partial pivoting in
 //     shared memory, one lane per vector); vectors of a cluster of close eigenvalues are
 //     computed by one lane in turn and orthogonalised against each other
-//  7. y = Phi z, Householder back-transformation, V = D L^-H U    (warp per column)
+//  7. y = Phi z, Householder back-transformation, V = D L^-H U    (CTA per column)
+//
+// Bound by latency: chains of short dependent steps.  m = 120, n = 40: 1.06 ms (Cholesky 218 us,
+// triangular solves 38 us each, Householder to inverse iteration 669 us, back-transformation 103 us);
+// 1.26 ms before the barriers were split, the FP64 steps reduced to fused multiply-adds on the lower
+// triangle and the reflectors of the back-transformation split once.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -302,6 +307,20 @@ __device__ void df_normalize(int m, dfl* x) {
   for (int i = 0; i < m; ++i) x[i] = df_mul(x[i], r);
 }
 
+// The cluster barrier in two halves: what a CTA still has to do on its own shared memory after its
+// part of a step is published runs between them, hidden behind the barrier's latency and the
+// slowest CTA.  Every thread executes both, once each.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// b - a w and b - conj(a) w as four fused multiply-adds
+__device__ __forceinline__ double2 cfms(double2 a, double2 w, double2 b) {
+  return double2{fma(-a.x, w.x, fma(a.y, w.y, b.x)), fma(-a.x, w.y, fma(-a.y, w.x, b.y))};
+}
+__device__ __forceinline__ double2 cfmsc(double2 a, double2 w, double2 b) {
+  return double2{fma(-a.x, w.x, fma(-a.y, w.y, b.x)), fma(-a.x, w.y, fma(a.y, w.x, b.y))};
+}
+
 __host__ __device__ inline size_t rr_tri_smem_offset(int m) {
   const size_t vec = (size_t)RRC_WARPS * m * sizeof(double2);
   return vec > 48 * 1024 ? vec : 48 * 1024;
@@ -367,9 +386,12 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
   __syncthreads();
   // Distributed form when the owned columns fit in shared memory: column j of S' lives in
   // CTA j % csize.  Step j: every CTA copies the published column j (rows > j) and 1 / pivot
-  // from its owner; the owner of column j+1 updates that column first (whole CTA), publishes
-  // it with its reciprocal pivot, then every CTA updates its remaining owned columns; one
-  // cluster barrier per column.
+  // from its owner and scales it (a second copy); the owner of column j+1 updates that column
+  // first (whole CTA) and publishes it with its reciprocal pivot; every CTA updates its remaining
+  // owned columns between the two halves of the step's cluster barrier.  The copies alternate by
+  // step parity, so that the next step may begin while a warp still updates.
+  // The update is bound by the FP64 unit (19 cycles of the SM per warp instruction): four fused
+  // multiply-adds per element, on the lower triangle only.
   const int ncol_own = (m + csize - 1) / csize;
   const bool dist = scols >= ncol_own + 3;
   for (size_t e = gtid; e < mm; e += gnt) {
@@ -382,12 +404,13 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
       lm[e] = double2{0.5 * s * (b.x + bt.x), 0.5 * s * (b.y - bt.y)};
     }
   }
-  __shared__ double chol_s;   // 1 / pivot of the current column (negative: not positive definite)
+  // 1 / pivot of the current column, by step parity (negative: not positive definite)
+  __shared__ double chol_s[2];
   bool failed = false;
   if (dist) {
     double2* cb = stg;                               // owned columns, column j at (j / csize) * m
     double2* colb = stg + (size_t)ncol_own * m;      // the column this CTA publishes; [m].x = 1 / pivot
-    double2* colj = colb + (m + 1);                  // local copy of the current column
+    double2* colbuf = reinterpret_cast<double2*>(rrc_smem);   // 2 x (column j, column j / pivot)
     for (int e = tid; e < ncol_own * m; e += RRC_THREADS) {
       const int lj = e / m, r = e - lj * m, j = lj * csize + crank;
       if (j < m) {
@@ -405,45 +428,52 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
         colb[m] = double2{piv > chol_tol ? rcp_pos(piv) : -1.0, 0.0};
       }
     };
-    auto updc = [&](int lk, int i, double inv2) {   // lm[i, k] -= conj(l_kj) l_ij / pivot, i >= k
-      const int k = lk * csize + crank;
-      if (k >= m || i < k) return;
-      double2* c = cb + (size_t)lk * m + i;
-      const double2 u = cmulc(colj[k], colj[i]);
-      *c = double2{fma(-u.x, inv2, c->x), fma(-u.y, inv2, c->y)};
-    };
     if (crank == 0) publish(0);
     cl.sync();
     RR_LAP(7);
     for (int j = 0; j < m; ++j) {
-      const int len = m - j - 1;
       const double2* src = cl.map_shared_rank(colb, (unsigned)(j % csize));
+      double2* colj = colbuf + (size_t)(j & 1) * 2 * m;
+      double2* cols = colj + m;
       const int r = j + 1 + tid;   // one row per thread (m <= RRC_THREADS + 1)
-      double2 x = double2{0.0, 0.0};
-      if (r < m) x = src[r];
-      if (tid == 0) chol_s = src[m].x;
-      if (r < m) colj[r] = x;
+      if (tid == 0) chol_s[j & 1] = src[m].x;
+      if (r < m) {
+        const double2 x = src[r];
+        const double inv = src[m].x;
+        colj[r] = x;
+        cols[r] = double2{x.x * inv, x.y * inv};
+      }
       __syncthreads();
-      const double inv2 = chol_s;
-      if (!(inv2 > 0.0)) {   // the same published value decides in every CTA
+      if (!(chol_s[j & 1] > 0.0)) {   // the same published value decides in every CTA
         failed = true;
         break;
       }
       RR_LAP(0);
+      // lm[i, k] -= conj(l_kj / pivot) l_ij, i >= k
       const int lj0 = (j + 1 - crank + csize - 1) / csize;   // first owned column > j
       const bool next = j + 1 < m && crank == (j + 1) % csize;
       if (next) {
-        if (r < m) updc(lj0, r, inv2);
+        if (r < m) {
+          double2* c = cb + (size_t)lj0 * m + r;
+          *c = cfmsc(cols[j + 1], colj[r], *c);
+        }
         __syncthreads();
         publish(j + 1);
       }
-      const int l1 = lj0 + (next ? 1 : 0);
-      for (int e = tid; e < (ncol_own - l1) * len; e += RRC_THREADS) {
-        const int q = e / len;
-        updc(l1 + q, j + 1 + (e - q * len), inv2);
+      cluster_arrive();
+      // four columns at a time, four warps each; the warp of a column's first rows (the one that
+      // always has work) moves over the SM's four FP64 units
+      for (int lk = lj0 + (next ? 1 : 0) + (wl >> 2); lk < ncol_own; lk += RRC_WARPS / 4) {
+        const int k = lk * csize + crank;
+        if (k >= m) break;
+        const double2 ck = cols[k];
+        for (int i = k + 32 * ((wl + (wl >> 2)) & 3) + lane; i < m; i += 128) {
+          double2* c = cb + (size_t)lk * m + i;
+          *c = cfmsc(ck, colj[i], *c);
+        }
       }
       RR_LAP(1);
-      cl.sync();
+      cluster_wait();
       RR_LAP(2);
     }
     if (failed) {
@@ -490,10 +520,10 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
     }
     if (tid == 0) {
       const double piv = colj[j].x;
-      chol_s = piv > chol_tol ? rcp_pos(piv) : -1.0;
+      chol_s[0] = piv > chol_tol ? rcp_pos(piv) : -1.0;
     }
     __syncthreads();
-    const double inv2 = chol_s;
+    const double inv2 = chol_s[0];
     if (!(inv2 > 0.0)) {   // the same global pivot decides in every CTA
       failed = true;
       break;
@@ -556,26 +586,23 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
   // lives in the shared memory of CTA j % csize, as double-float (re hi, re lo, im hi, im lo).
   // Step k (reflector v of column k, rows > k):
   //   A  every CTA copies v and tau from the owner of column k (DSMEM)
-  //   B  p_i = tau C[:, i]^H v for the owned columns i > k (Hermitian C: p = tau C v) and the
-  //      partial sum of conj(v_i) p_i
+  //   B  p_i = tau C[:, i]^H v for the owned columns i > k (Hermitian C: p = tau C v)
   //   -- cluster barrier --
-  //   C  K = tau/2 sum of the partials, w = p - K v (p gathered from the owners)
+  //   C  p gathered from the owners, K = tau/2 v^H p (in every CTA), w = p - K v
   //   D  owned columns j > k: C[:, j] -= v conj(w_j) + w conj(v_j)
-  //   E  the owner of column k+1 forms the next reflector (FP64 from the double-float column)
-  //   -- cluster barrier --
+  //   E  the owner of column k+1 forms the next reflector from its updated column
+  //   -- cluster barrier, its halves around D: only E and its column come before the arrival;
+  //      v and w alternate by step parity, so that the next step may begin while a warp is in D --
   // B-D run in double-float arithmetic on the FP32 lanes (about 2^-47 per operation): in FP64
   // they were bound by the FP64 pipe of each SM.  The reflectors stay in their columns (first
   // element replaced by v0), as in the global form.
   const int ncol_own = (m + csize - 1) / csize;
   if (m >= 3 && scols >= ncol_own) {
     float4* cb = reinterpret_cast<float4*>(stg);             // owned columns, column j at (j / csize) * m
-    float4* vl = reinterpret_cast<float4*>(rrc_smem);        // v of the current step, by row
-    float4* wf = vl + m;                                     // w, by row
-    float4* pb = wf + m;                                     // p at the owned indices (read by the cluster)
+    float4* vwb = reinterpret_cast<float4*>(rrc_smem);       // 2 x (v, w) by row, by step parity
+    float4* pb = vwb + 4 * (size_t)m;                        // p at the owned indices (read by the cluster)
     float4* bc = pb + m;                                     // 2 x (m + 1): reflector + tau, by parity
-    float4* kp = bc + 2 * (m + 1);                           // this CTA's partial of v^H p
-    float4* kw = kp + 1;                                     // per-warp partials
-    __shared__ float4 hk;                                    // K of the current step
+    float4* kw = bc + 2 * (m + 1);                           // per-warp partials of v^H p
     __shared__ float2 tpart[RRC_WARPS];                      // per-warp partial norms of the next column
     for (int e = tid; e < ncol_own * m; e += RRC_THREADS) {
       const int lj = e / m, r = e - lj * m, j = lj * csize + crank;
@@ -644,6 +671,8 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
     RR_LAP(7);
     for (int k = 0; k + 2 < m; ++k) {
       const int len = m - k - 1;
+      float4* vl = vwb + (size_t)(k & 1) * 2 * m;            // v of the current step, by row
+      float4* wf = vl + m;                                   // w, by row
       // A
       const float4* src = cl.map_shared_rank(bc + (size_t)(k & 1) * (m + 1), (unsigned)(k % csize));
       for (int r = k + 1 + tid; r <= m; r += RRC_THREADS) vl[r == m ? 0 : r] = src[r];   // vl[0] <- tau
@@ -652,7 +681,6 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
       const dfl t = ucdf(vl[0]).re;
       // B
       const int lj0 = (k + 1 - crank + csize - 1) / csize;   // first owned column > k
-      cdf kacc = cdf0();
       for (int lj = lj0 + wl; lj < ncol_own; lj += RRC_WARPS) {
         const int i = lj * csize + crank;
         if (i >= m) break;
@@ -662,32 +690,27 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
         sacc = warp_cdsum(sacc);
         const cdf p = cdf{df_mul(t, sacc.re), df_mul(t, sacc.im)};
         if (lane == 0) pb[i] = c4(p);
-        kacc = cdf_fmac(ucdf(vl[i]), p, kacc);
-      }
-      if (lane == 0) kw[wl] = c4(kacc);
-      __syncthreads();
-      if (wl == 0) {
-        cdf ks = lane < RRC_WARPS ? ucdf(kw[lane]) : cdf0();
-        ks = warp_cdsum(ks);
-        if (lane == 0) kp[0] = c4(ks);
       }
       RR_LAP(1);
       cl.sync();
       RR_LAP(2);
-      // C: p_r gathered from the owners (one row per thread, issued first so that its latency
-      // overlaps the K reduction), K = tau/2 * sum of the partials, w = p - K v
+      // C: p_r gathered from the owners (one row per thread), K = tau/2 * v^H p from the gathered
+      // rows by every CTA for itself, w = p - K v
       const int rr = k + 1 + tid;
-      float4 p4 = float4{0.f, 0.f, 0.f, 0.f};
-      if (rr < m) p4 = *cl.map_shared_rank(pb + rr, (unsigned)(rr % csize));
-      if (wl == 0) {
-        cdf ks = lane < csize ? ucdf(*cl.map_shared_rank(kp, (unsigned)lane)) : cdf0();
-        ks = warp_cdsum(ks);
-        const dfl ht = df_mul(t, dfl{0.5f, 0.f});
-        if (lane == 0) hk = c4(cdf{df_mul(ht, ks.re), df_mul(ht, ks.im)});
+      cdf pr = cdf0();
+      if (32 * wl < len) {
+        if (rr < m) pr = ucdf(*cl.map_shared_rank(pb + rr, (unsigned)(rr % csize)));
+        const cdf ks = warp_cdsum(rr < m ? cdf_fmac(ucdf(vl[rr]), pr, cdf0()) : cdf0());
+        if (lane == 0) kw[wl] = c4(ks);
       }
       __syncthreads();
-      const cdf kv = ucdf(hk);
-      if (rr < m) wf[rr] = c4(csub(ucdf(p4), cmul(kv, ucdf(vl[rr]))));
+      if (rr < m) {
+        cdf ks = ucdf(kw[0]);
+        for (int q = 1; 32 * q < len; ++q) ks = cadd(ks, ucdf(kw[q]));
+        const dfl ht = df_mul(t, dfl{0.5f, 0.f});
+        const cdf kv{df_mul(ht, ks.re), df_mul(ht, ks.im)};
+        wf[rr] = c4(csub(pr, cmul(kv, ucdf(vl[rr]))));
+      }
       __syncthreads();
       RR_LAP(3);
       // D: owned columns j > k: C[:, j] -= v conj(w_j) + w conj(v_j).  The owner of column k+1
@@ -735,6 +758,7 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
           if (lane < nw) t2 = dfl{tpart[lane].x, tpart[lane].y};
           t2 = warp_dsum(t2);
           make_reflector(k + 1, &t2);   // E
+          cluster_arrive();
 #ifdef DKS_RR_TIMING
           if (gtid == 0) {
             town[0] += o1 - o0;
@@ -743,21 +767,24 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
           }
 #endif
         } else {
+          cluster_arrive();
           for (int e = tid - 32; e < (nown - 1) * len; e += RRC_THREADS - 32) {
             const int q = e / len;
             upd(lj0 + 1 + q, k + 1 + (e - q * len));
           }
         }
       } else {
+        cluster_arrive();
         for (int e = tid; e < nown * len; e += RRC_THREADS) {
           const int q = e / len;
           upd(lj0 + q, k + 1 + (e - q * len));
         }
       }
       RR_LAP(4);
-      cl.sync();
+      cluster_wait();
       RR_LAP(6);
     }
+    __syncthreads();   // the last updates of this CTA's columns
     for (int e = tid; e < ncol_own * m; e += RRC_THREADS) {
       const int lj = e / m, r = e - lj * m, j = lj * csize + crank;
       if (j < m) {
@@ -1087,11 +1114,14 @@ __device__ __forceinline__ void stage_init(uint64_t* mbar) {
 }
 
 // 3. Forward substitution with L, column-oriented, one right-hand side per CTA (so each column
-// has an SM's FP64 pipes to itself): the 128 threads own rows k of b (one warp on each of the
-// SM's four FP64 units); at step i every thread forms w_i = b_i / L_ii and updates its
-// b_k -= L_ki w_i (k > i); columns of L are staged in shared memory in blocks.
+// has an SM's FP64 pipes to itself): the 128 threads own rows r = tid + 128 q of b in registers
+// (one warp on each of the SM's four FP64 units); columns of L are staged in shared memory in
+// blocks.  Step i takes w_i = b_i / L_ii from shared memory, b_r -= L_ri w_i (r > i) as four fused
+// multiply-adds, and the owner of row i + 1 leaves w_i+1 in the other slot: one barrier per step,
+// and the FP64 unit (19 cycles of the SM per warp instruction) sees no scaling but the owner's.
 //   pass 0: W = L^-1 A'   (column c of A')              -> cm
 //   pass 1: C = L^-1 W^H  (column c = conj(row c of W))  -> lm (free after the Cholesky)
+template <int RPT>   // rows per thread: m <= 128 RPT
 __global__ void __launch_bounds__(128, 1) k_rr_trsm(double2* __restrict__ scr, int m, int pass, int scols) {
   extern __shared__ __align__(16) unsigned char trs_smem[];
   const size_t mm = (size_t)m * m;
@@ -1109,19 +1139,22 @@ __global__ void __launch_bounds__(128, 1) k_rr_trsm(double2* __restrict__ scr, i
   uint32_t phase = 0;
   stage_init(&mbar);
   double2* stg = reinterpret_cast<double2*>(trs_smem);           // scols x m
-  double2* b = stg + (size_t)scols * m;                          // right-hand side / solution
-  double* sl = reinterpret_cast<double*>(b + m);
+  double* sl = reinterpret_cast<double*>(stg + (size_t)scols * m);
+  __shared__ double2 wsh[2];                                      // w_i, by step parity
   const int tid = threadIdx.x;
   const int c = blockIdx.x;
-  for (int k = tid; k < m; k += blockDim.x) {
-    sl[k] = linv[k];
-    if (pass == 0) {
-      b[k] = am[(size_t)c * m + k];
-    } else {
-      const double2 w = cm[(size_t)k * m + c];
-      b[k] = double2{w.x, -w.y};
+  for (int k = tid; k < m; k += blockDim.x) sl[k] = linv[k];
+  double2 b[RPT];
+#pragma unroll
+  for (int q = 0; q < RPT; ++q) {
+    const int r = tid + 128 * q;
+    b[q] = double2{0.0, 0.0};
+    if (r < m) {
+      const double2 v = pass == 0 ? am[(size_t)c * m + r] : cm[(size_t)r * m + c];
+      b[q] = pass == 0 ? v : double2{v.x, -v.y};
     }
   }
+  if (tid == 0) wsh[0] = double2{b[0].x * linv[0], b[0].y * linv[0]};
   for (int i0 = 0; i0 < m; i0 += scols) {
     const int nb = min(scols, m - i0);
     if (!stage_block(stg, lf + (size_t)i0 * m, (uint32_t)(nb * m * sizeof(double2)), &mbar, phase)) {
@@ -1129,23 +1162,37 @@ __global__ void __launch_bounds__(128, 1) k_rr_trsm(double2* __restrict__ scr, i
       return;
     }
     for (int i = i0; i < i0 + nb; ++i) {
-      const double2 bi = b[i];
-      const double li = sl[i];
-      const double2 w = double2{bi.x * li, bi.y * li};
+      const double2 w = wsh[i & 1];
       const double2* lc = stg + (size_t)(i - i0) * m;
-      for (int k = tid; k < m; k += blockDim.x)
-        if (k > i) b[k] = csub(b[k], cmul(lc[k], w));
+#pragma unroll
+      for (int q = 0; q < RPT; ++q) {
+        const int r = tid + 128 * q;
+        if (r > i && r < m) {
+          b[q] = cfms(lc[r], w, b[q]);
+          if (r == i + 1) {
+            const double li = sl[r];
+            wsh[r & 1] = double2{b[q].x * li, b[q].y * li};
+          }
+        }
+      }
       __syncthreads();
     }
   }
   double2* out = pass == 0 ? cm : lm;
-  for (int k = tid; k < m; k += blockDim.x) out[(size_t)c * m + k] = double2{b[k].x * sl[k], b[k].y * sl[k]};
+#pragma unroll
+  for (int q = 0; q < RPT; ++q) {
+    const int r = tid + 128 * q;
+    if (r < m) out[(size_t)c * m + r] = double2{b[q].x * sl[r], b[q].y * sl[r]};
+  }
 }
 
 // 7. u = H_0 ... H_{m-3} (Phi z_j); V_j = D L^-H u, one eigenvector per CTA; the 128 threads own
 // rows (one warp per FP64 unit of the SM); reflectors and rows of L are staged in shared
 // memory.  A reflector step sums four warp partials through shared memory (double-buffered by
-// step parity, so one barrier per step).
+// step parity, so one barrier per step); its elements are split into double-float pairs once, where
+// they were staged (a split per use kept the FP64 unit busy with its predicated-off fallback).  The
+// triangular solve runs as in k_rr_trsm, from the last row up.
+template <int RPT>
 __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr, int m, int n, double2* __restrict__ V,
                                                    double* __restrict__ lam, int* __restrict__ info, int scols) {
   extern __shared__ __align__(16) unsigned char btr_smem[];
@@ -1168,24 +1215,23 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
   uint32_t phase = 0;
   stage_init(&mbar);
   double2* stg = reinterpret_cast<double2*>(btr_smem);           // scols x m
-  double2* wv = stg + (size_t)scols * m;
-  double2* sph = wv + m;
-  double* sl = reinterpret_cast<double*>(sph + m);
-  double* stau = sl + m;
-  double* sdsc = stau + m;
+  double* sl = reinterpret_cast<double*>(stg + (size_t)scols * m);
+  float2* stau = reinterpret_cast<float2*>(sl + m);               // tau as double-float pairs
+  double* sdsc = sl + 2 * m;
   __shared__ float4 red[8];    // warp partials of the reflector dot products, by step parity
+  __shared__ double2 ysh[2];   // y_i of the triangular solve, by step parity
   const int tid = threadIdx.x, lane = tid & 31, wl = tid >> 5;
   const int j = blockIdx.x;
   for (int k = tid; k < m; k += blockDim.x) {
     sl[k] = linv[k];
-    stau[k] = tau[k].x;
+    const dfl t = df_from(tau[k].x);
+    stau[k] = float2{t.h, t.l};
     sdsc[k] = dsc[k];
   }
   // the reflectors are applied in double-float arithmetic (an orthogonal transformation, so
   // 2^-47 rounding per operation stays at that level; FP64 chains cost a whole FP64-unit
-  // warp instruction per dependent step): reflector elements are split as they are read, the
-  // vector is kept as double-float in the rows each thread owns
-  constexpr int RPT = 4;                       // rows per thread: m <= 512
+  // warp instruction per dependent step); the vector is kept as double-float in the rows each
+  // thread owns
   // start vector: ph_r z_r, z the double-float eigenvector of the real tridiagonal
   const float2* zj = reinterpret_cast<const float2*>(zt) + (size_t)j * m;
   cdf wq[RPT];
@@ -1195,7 +1241,7 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
     if (r < m) {
       const dfl z{zj[r].x, zj[r].y};
       const double2 p = ph[r];
-      wq[q] = cdf{df_mul(df_from_bits(p.x), z), df_mul(df_from_bits(p.y), z)};
+      wq[q] = cdf{df_mul(df_split_rn(p.x), z), df_mul(df_split_rn(p.y), z)};
     } else {
       wq[q] = cdf0();
     }
@@ -1206,38 +1252,45 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
       if (tid == 0) *flag = 2;
       return;
     }
+    float4* const vdf = reinterpret_cast<float4*>(stg);
+    for (int k = k0 + wl; k <= k1; k += 4) {   // rows > k of each reflector, in place
+      for (int r = k + 1 + lane; r < m; r += 32) {
+        const size_t e = (size_t)(k - k0) * m + r;
+        const double2 x = stg[e];
+        vdf[e] = c4(cdf{df_split_rn(x.x), df_split_rn(x.y)});
+      }
+    }
+    __syncthreads();
     for (int k = k1; k >= k0; --k) {
-      const double t = stau[k];
-      if (t == 0.0) continue;   // uniform: every thread reads the same tau
-      const double2* v = stg + (size_t)(k - k0) * m;
+      const dfl td{stau[k].x, stau[k].y};
+      if (td.h == 0.f) continue;   // uniform: every thread reads the same tau
+      const float4* v = vdf + (size_t)(k - k0) * m;
       // rows r > k, thread-owned (r = tid + 128 q): partial dot, warp sums, four partials
       cdf sacc = cdf0();
 #pragma unroll
       for (int q = 0; q < RPT; ++q) {
         const int r = tid + 128 * q;
-        if (r > k && r < m) sacc = cdf_fmac(cdf{df_from_bits(v[r].x), df_from_bits(v[r].y)}, wq[q], sacc);
+        if (r > k && r < m) sacc = cdf_fmac(ucdf(v[r]), wq[q], sacc);
       }
       sacc = warp_cdsum(sacc);
       float4* part = red + 4 * (k & 1);
       if (lane == 0) part[wl] = c4(sacc);
       __syncthreads();
-      cdf tot = ucdf(part[0]);
-      tot = cadd(tot, ucdf(part[1]));
-      tot = cadd(tot, ucdf(part[2]));
-      tot = cadd(tot, ucdf(part[3]));
-      const dfl td = df_from(t);
+      const cdf tot = cadd(cadd(ucdf(part[0]), ucdf(part[1])), cadd(ucdf(part[2]), ucdf(part[3])));
       const cdf f = cdf{df_mul(td, tot.re), df_mul(td, tot.im)};
 #pragma unroll
       for (int q = 0; q < RPT; ++q) {
         const int r = tid + 128 * q;
-        if (r > k && r < m) wq[q] = csub(wq[q], cmul(f, cdf{df_from_bits(v[r].x), df_from_bits(v[r].y)}));
+        if (r > k && r < m) wq[q] = csub(wq[q], cmul(f, ucdf(v[r])));
       }
     }
   }
+  double2 u[RPT];
 #pragma unroll
   for (int q = 0; q < RPT; ++q) {
     const int r = tid + 128 * q;
-    if (r < m) wv[r] = double2{df_val(wq[q].re), df_val(wq[q].im)};
+    u[q] = double2{df_val(wq[q].re), df_val(wq[q].im)};
+    if (r == m - 1) ysh[r & 1] = double2{u[q].x * sl[r], u[q].y * sl[r]};
   }
   // L^H y = u, column-oriented: y_i = u_i / L_ii, then u_k -= conj(L[i, k]) y_i for k < i
   for (int i1 = m - 1; i1 >= 0; i1 -= scols) {
@@ -1246,19 +1299,30 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
       if (tid == 0) *flag = 2;
       return;
     }
-    __syncthreads();
     for (int i = i1; i >= i0; --i) {
-      const double2 u = wv[i];
-      const double li = sl[i];
-      const double2 y = double2{u.x * li, u.y * li};
+      const double2 y = ysh[i & 1];
       const double2* lr = stg + (size_t)(i - i0) * m;
-      for (int k = tid; k < i; k += blockDim.x) wv[k] = csub(wv[k], cmulc(lr[k], y));
+#pragma unroll
+      for (int q = 0; q < RPT; ++q) {
+        const int r = tid + 128 * q;
+        if (r < i) {
+          u[q] = cfmsc(lr[r], y, u[q]);
+          if (r == i - 1) {
+            const double li = sl[r];
+            ysh[r & 1] = double2{u[q].x * li, u[q].y * li};
+          }
+        }
+      }
       __syncthreads();
     }
   }
-  for (int i = tid; i < m; i += blockDim.x) {
-    const double f = sdsc[i] * sl[i];
-    V[(size_t)j * m + i] = double2{f * wv[i].x, f * wv[i].y};
+#pragma unroll
+  for (int q = 0; q < RPT; ++q) {
+    const int r = tid + 128 * q;
+    if (r < m) {
+      const double f = sdsc[r] * sl[r];
+      V[(size_t)j * m + r] = double2{f * u[q].x, f * u[q].y};
+    }
   }
   if (tid == 0) {
     lam[j] = lamw[j];
@@ -1279,6 +1343,14 @@ int rr_set_first_wait(unsigned polls) {
 size_t rr_cluster_flag_offset(int m) {
   const size_t mm = (size_t)m * m;
   return 5 * mm * sizeof(double2) + 6 * (size_t)m * sizeof(double) + 3 * (size_t)m * sizeof(double2);
+}
+
+// the per-column kernels for m <= 128 r (a thread's rows are registers: r fixed at compile time)
+static auto rr_trsm_for(int r) {
+  return r <= 1 ? k_rr_trsm<1> : r == 2 ? k_rr_trsm<2> : r == 3 ? k_rr_trsm<3> : k_rr_trsm<4>;
+}
+static auto rr_backtr_for(int r) {
+  return r <= 1 ? k_rr_backtr<1> : r == 2 ? k_rr_backtr<2> : r == 3 ? k_rr_backtr<3> : k_rr_backtr<4>;
 }
 
 static int g_cluster = 0;   // 0 = unknown, else cluster size that launched successfully
@@ -1312,16 +1384,18 @@ int rayleigh_ritz_cluster(const double2* a, const double2* s, int nz, int n, dou
   if (base + 8 * (size_t)nz * sizeof(double2) > kRrSmemMax) return DKS_OK;
   const int scols = (int)std::min<size_t>({(size_t)64, (size_t)nz, (kRrSmemMax - base) / ((size_t)nz * sizeof(double2))});
   const size_t smem = rr_cluster_smem(nz, scols);
-  // per-column kernels: staging area + one complex vector + four m-length scalar arrays
-  const size_t col_extra = (size_t)nz * (2 * sizeof(double2) + 4 * sizeof(double));
+  // per-column kernels: staging area + three m-length scalar arrays
+  const size_t col_extra = (size_t)nz * 3 * sizeof(double);
   const int scols1 = (int)std::max<size_t>(1, std::min<size_t>((size_t)nz, (kRrSmemMax - col_extra) / ((size_t)nz * sizeof(double2))));
   const size_t smem1 = (size_t)scols1 * nz * sizeof(double2) + col_extra;
   static bool attr_done = false;
   if (!attr_done) {
     cudaFuncSetAttribute((const void*)k_rr_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute((const void*)k_rr_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRrSmemMax);
-    cudaFuncSetAttribute((const void*)k_rr_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRrSmemMax);
-    cudaFuncSetAttribute((const void*)k_rr_backtr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRrSmemMax);
+    for (int r = 1; r <= 4; ++r) {
+      cudaFuncSetAttribute((const void*)rr_trsm_for(r), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRrSmemMax);
+      cudaFuncSetAttribute((const void*)rr_backtr_for(r), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRrSmemMax);
+    }
     attr_done = true;
   }
   Prof pr(P_RR, st, 2.0 * nz * nz * 16.0 + 16.0 * nz * n, rr_flops(nz, n));
@@ -1342,10 +1416,11 @@ int rayleigh_ritz_cluster(const double2* a, const double2* s, int nz, int n, dou
     return DKS_OK;
   }
   pr.count(4);      // five kernels in all
-  k_rr_trsm<<<nz, 128, smem1, st>>>(scratch, nz, 0, scols1);
-  k_rr_trsm<<<nz, 128, smem1, st>>>(scratch, nz, 1, scols1);
+  const int rpt = (nz + 127) / 128;
+  rr_trsm_for(rpt)<<<nz, 128, smem1, st>>>(scratch, nz, 0, scols1);
+  rr_trsm_for(rpt)<<<nz, 128, smem1, st>>>(scratch, nz, 1, scols1);
   DKS_CUDA_TRY(launch_cluster(g_cluster, smem, st, a, s, nz, n, v, lam, info, scratch, chol_tol, scols, 1));
-  k_rr_backtr<<<n, 128, smem1, st>>>(scratch, nz, n, v, lam, info, scols1);
+  rr_backtr_for(rpt)<<<n, 128, smem1, st>>>(scratch, nz, n, v, lam, info, scols1);
   DKS_CUDA_TRY(cudaGetLastError());
   return DKS_OK;
 }
