@@ -24,10 +24,11 @@
 //     computed by one lane in turn and orthogonalised against each other
 //  7. y = Phi z, Householder back-transformation, V = D L^-H U    (CTA per column)
 //
-// Bound by latency: chains of short dependent steps.  m = 120, n = 40: 1.06 ms (Cholesky 218 us,
-// triangular solves 38 us each, Householder to inverse iteration 669 us, back-transformation 103 us);
-// 1.26 ms before the barriers were split, the FP64 steps reduced to fused multiply-adds on the lower
-// triangle and the reflectors of the back-transformation split once.
+// Bound by latency: chains of short dependent steps.  m = 120, n = 40: 992 us in all.  1.26 ms
+// before the barriers were split, the FP64 steps reduced to fused multiply-adds on the lower triangle
+// and the reflectors of the back-transformation split once (1059 us: Cholesky 218, triangular solves
+// 38 each, Householder to inverse iteration 669, back-transformation 103), and the columns, reflectors
+// and p written into every CTA instead of read from their owners (992 us).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -385,11 +386,12 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
   }
   __syncthreads();
   // Distributed form when the owned columns fit in shared memory: column j of S' lives in
-  // CTA j % csize.  Step j: every CTA copies the published column j (rows > j) and 1 / pivot
-  // from its owner and scales it (a second copy); the owner of column j+1 updates that column
-  // first (whole CTA) and publishes it with its reciprocal pivot; every CTA updates its remaining
-  // owned columns between the two halves of the step's cluster barrier.  The copies alternate by
-  // step parity, so that the next step may begin while a warp still updates.
+  // CTA j % csize.  Step j: every CTA has column j (rows > j) and 1 / pivot from its owner and
+  // scales it (a second copy); the owner of column j+1 updates that column first (whole CTA) and
+  // writes it and its reciprocal pivot into every CTA (a read from the owner would wait for a
+  // round trip at the start of each step); every CTA updates its remaining owned columns between the
+  // two halves of the step's cluster barrier.  Three copies in turn: while the owner writes column
+  // j+1, a warp elsewhere may still update with column j-1.
   // The update is bound by the FP64 unit (19 cycles of the SM per warp instruction): four fused
   // multiply-adds per element, on the lower triangle only.
   const int ncol_own = (m + csize - 1) / csize;
@@ -404,13 +406,12 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
       lm[e] = double2{0.5 * s * (b.x + bt.x), 0.5 * s * (b.y - bt.y)};
     }
   }
-  // 1 / pivot of the current column, by step parity (negative: not positive definite)
-  __shared__ double chol_s[2];
+  __shared__ double chol_s;   // 1 / pivot of the current column (negative: not positive definite)
   bool failed = false;
   if (dist) {
     double2* cb = stg;                               // owned columns, column j at (j / csize) * m
-    double2* colb = stg + (size_t)ncol_own * m;      // the column this CTA publishes; [m].x = 1 / pivot
-    double2* colbuf = reinterpret_cast<double2*>(rrc_smem);   // 2 x (column j, column j / pivot)
+    // 3 x (column j and at [m].x 1 / pivot, written by the owner; column j / pivot)
+    double2* colbuf = reinterpret_cast<double2*>(rrc_smem);
     for (int e = tid; e < ncol_own * m; e += RRC_THREADS) {
       const int lj = e / m, r = e - lj * m, j = lj * csize + crank;
       if (j < m) {
@@ -422,29 +423,30 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
     __syncthreads();
     auto publish = [&](int j) {   // whole CTA; column j is owned here and final
       const double2* cj = cb + (size_t)(j / csize) * m;
-      for (int i = j + 1 + tid; i < m; i += RRC_THREADS) colb[i] = cj[i];
-      if (tid == 0) {
+      double2* dst = colbuf + (size_t)(j % 3) * (2 * m + 1);
+      if (wl == 0) {
         const double piv = cj[j].x;
-        colb[m] = double2{piv > chol_tol ? rcp_pos(piv) : -1.0, 0.0};
+        const double inv = piv > chol_tol ? rcp_pos(piv) : -1.0;
+        if (lane < csize) cl.map_shared_rank(dst, (unsigned)lane)[m] = double2{inv, 0.0};
+      } else {
+        for (int c = wl - 1; c < csize; c += RRC_WARPS - 1) {
+          double2* d = cl.map_shared_rank(dst, (unsigned)c);
+          for (int i = j + 1 + lane; i < m; i += 32) d[i] = cj[i];
+        }
       }
     };
+    cl.sync();   // every CTA runs: its shared memory may be written
     if (crank == 0) publish(0);
     cl.sync();
     RR_LAP(7);
     for (int j = 0; j < m; ++j) {
-      const double2* src = cl.map_shared_rank(colb, (unsigned)(j % csize));
-      double2* colj = colbuf + (size_t)(j & 1) * 2 * m;
-      double2* cols = colj + m;
+      const double2* colj = colbuf + (size_t)(j % 3) * (2 * m + 1);
+      double2* cols = colbuf + (size_t)(j % 3) * (2 * m + 1) + (m + 1);
       const int r = j + 1 + tid;   // one row per thread (m <= RRC_THREADS + 1)
-      if (tid == 0) chol_s[j & 1] = src[m].x;
-      if (r < m) {
-        const double2 x = src[r];
-        const double inv = src[m].x;
-        colj[r] = x;
-        cols[r] = double2{x.x * inv, x.y * inv};
-      }
+      const double inv = colj[m].x;
+      if (r < m) cols[r] = double2{colj[r].x * inv, colj[r].y * inv};
       __syncthreads();
-      if (!(chol_s[j & 1] > 0.0)) {   // the same published value decides in every CTA
+      if (!(inv > 0.0)) {   // the same published value decides in every CTA
         failed = true;
         break;
       }
@@ -520,10 +522,10 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
     }
     if (tid == 0) {
       const double piv = colj[j].x;
-      chol_s[0] = piv > chol_tol ? rcp_pos(piv) : -1.0;
+      chol_s = piv > chol_tol ? rcp_pos(piv) : -1.0;
     }
     __syncthreads();
-    const double inv2 = chol_s[0];
+    const double inv2 = chol_s;
     if (!(inv2 > 0.0)) {   // the same global pivot decides in every CTA
       failed = true;
       break;
@@ -585,10 +587,11 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
   // Distributed form (when the staging area holds this CTA's share of the columns): column j
   // lives in the shared memory of CTA j % csize, as double-float (re hi, re lo, im hi, im lo).
   // Step k (reflector v of column k, rows > k):
-  //   A  every CTA copies v and tau from the owner of column k (DSMEM)
-  //   B  p_i = tau C[:, i]^H v for the owned columns i > k (Hermitian C: p = tau C v)
+  //   A  v and tau are in every CTA, written by the owner of column k (DSMEM; reading them from the
+  //      owner would wait for a round trip here, and once more for p)
+  //   B  p_i = tau C[:, i]^H v for the owned columns i > k (Hermitian C: p = tau C v), into every CTA
   //   -- cluster barrier --
-  //   C  p gathered from the owners, K = tau/2 v^H p (in every CTA), w = p - K v
+  //   C  K = tau/2 v^H p (in every CTA), w = p - K v
   //   D  owned columns j > k: C[:, j] -= v conj(w_j) + w conj(v_j)
   //   E  the owner of column k+1 forms the next reflector from its updated column
   //   -- cluster barrier, its halves around D: only E and its column come before the arrival;
@@ -600,16 +603,23 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
   if (m >= 3 && scols >= ncol_own) {
     float4* cb = reinterpret_cast<float4*>(stg);             // owned columns, column j at (j / csize) * m
     float4* vwb = reinterpret_cast<float4*>(rrc_smem);       // 2 x (v, w) by row, by step parity
-    float4* pb = vwb + 4 * (size_t)m;                        // p at the owned indices (read by the cluster)
-    float4* bc = pb + m;                                     // 2 x (m + 1): reflector + tau, by parity
-    float4* kw = bc + 2 * (m + 1);                           // per-warp partials of v^H p
+    float4* pb = vwb + 4 * (size_t)m;                        // p by row, from the owners
+    float4* kw = pb + m;                                     // per-warp partials of v^H p
     __shared__ float2 tpart[RRC_WARPS];                      // per-warp partial norms of the next column
     for (int e = tid; e < ncol_own * m; e += RRC_THREADS) {
       const int lj = e / m, r = e - lj * m, j = lj * csize + crank;
       if (j < m) cb[e] = c4(cm[(size_t)j * m + r]);
     }
     __syncthreads();
-    // reflector of column k by warp 0 of its owner: broadcast buffer, v0 into the column, tau/ph.
+    // the rest of that reflector, the rows below its first, into every CTA: the owner's other warps
+    auto send_rows = [&](int k) {
+      const float4* x = cb + (size_t)(k / csize) * m;
+      for (int c = wl - 1; c < csize; c += RRC_WARPS - 1) {
+        float4* out = cl.map_shared_rank(vwb + (size_t)(k & 1) * 2 * m, (unsigned)c);
+        for (int r = k + 2 + lane; r < m; r += 32) out[r] = x[r];
+      }
+    };
+    // reflector of column k by warp 0 of its owner: v0 and tau into every CTA, v0 into the column, tau/ph.
     // All scalars in double-float on the FP32 lanes (a chain of FP64 operations here was the
     // critical path of every step); tau[k] and ph[k] are left as double-float quadruples in
     // their double2 slots and converted after the loop.
@@ -655,28 +665,30 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
           v0 = x0;
         }
       }
-      float4* out = bc + (size_t)(k & 1) * (m + 1);
       const float4 v04 = c4(v0);
-      for (int i = lane; i < len; i += 32) out[k + 1 + i] = i == 0 ? v04 : x[i];
+      if (lane < csize) {   // row 0 is in no reflector: tau
+        float4* out = cl.map_shared_rank(vwb + (size_t)(k & 1) * 2 * m, (unsigned)lane);
+        out[k + 1] = v04;
+        out[0] = float4{t.h, t.l, 0.f, 0.f};
+      }
       __syncwarp();
       if (lane == 0) {
-        out[m] = float4{t.h, t.l, 0.f, 0.f};
         if (t.h != 0.f) x[0] = v04;
         reinterpret_cast<float4*>(tau)[k] = float4{t.h, t.l, 0.f, 0.f};
         reinterpret_cast<float4*>(ph)[k] = c4(beta);
       }
     };
-    if (crank == 0 && wl == 0) make_reflector(0, nullptr);
+    if (crank == 0) {
+      if (wl == 0) make_reflector(0, nullptr);
+      else send_rows(0);
+    }
     cl.sync();
     RR_LAP(7);
     for (int k = 0; k + 2 < m; ++k) {
       const int len = m - k - 1;
       float4* vl = vwb + (size_t)(k & 1) * 2 * m;            // v of the current step, by row
       float4* wf = vl + m;                                   // w, by row
-      // A
-      const float4* src = cl.map_shared_rank(bc + (size_t)(k & 1) * (m + 1), (unsigned)(k % csize));
-      for (int r = k + 1 + tid; r <= m; r += RRC_THREADS) vl[r == m ? 0 : r] = src[r];   // vl[0] <- tau
-      __syncthreads();
+      __syncthreads();   // D of the step before, in this CTA
       RR_LAP(0);
       const dfl t = ucdf(vl[0]).re;
       // B
@@ -689,17 +701,16 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
         for (int r = k + 1 + lane; r < m; r += 32) sacc = cdf_fmac(ucdf(ci[r]), ucdf(vl[r]), sacc);
         sacc = warp_cdsum(sacc);
         const cdf p = cdf{df_mul(t, sacc.re), df_mul(t, sacc.im)};
-        if (lane == 0) pb[i] = c4(p);
+        if (lane < csize) *cl.map_shared_rank(pb + i, (unsigned)lane) = c4(p);
       }
       RR_LAP(1);
       cl.sync();
       RR_LAP(2);
-      // C: p_r gathered from the owners (one row per thread), K = tau/2 * v^H p from the gathered
-      // rows by every CTA for itself, w = p - K v
+      // C: K = tau/2 v^H p by every CTA for itself (one row per thread), w = p - K v
       const int rr = k + 1 + tid;
       cdf pr = cdf0();
       if (32 * wl < len) {
-        if (rr < m) pr = ucdf(*cl.map_shared_rank(pb + rr, (unsigned)(rr % csize)));
+        if (rr < m) pr = ucdf(pb[rr]);
         const cdf ks = warp_cdsum(rr < m ? cdf_fmac(ucdf(vl[rr]), pr, cdf0()) : cdf0());
         if (lane == 0) kw[wl] = c4(ks);
       }
@@ -767,6 +778,7 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
           }
 #endif
         } else {
+          send_rows(k + 1);
           cluster_arrive();
           for (int e = tid - 32; e < (nown - 1) * len; e += RRC_THREADS - 32) {
             const int q = e / len;
