@@ -9,8 +9,8 @@
 // 3D transform of one field (band, comp) runs in three passes that keep all
 // intermediates in a stick-compressed buffer T[field][p3][stick] sized to stay
 // resident in the 129 MB L2:
-//   pass A  scatter the stick into a zeroed length-N3 line in shared memory,
-//           inverse FFT along axis 3 (DIF, natural in -> digit-reversed out)
+//   pass A  the stick's consecutive planewaves, and zeros, into a length-N3 line in shared memory,
+//           inverse FFT along axis 3 (DIF, natural in -> digit-reversed out) whose last pass stores to T
 //   pass B  one (field, plane) per CTA: scatter the sticks into an N1 x N2 plane
 //           in shared memory, inverse 2D FFT (DIF), multiply by V/Ng stored in
 //           the same digit-reversed order, forward 2D FFT (DIT, digit-reversed in
