@@ -1200,8 +1200,8 @@ __global__ void __launch_bounds__(128, 1) k_rr_trsm(double2* __restrict__ scr, i
 
 // 7. u = H_0 ... H_{m-3} (Phi z_j); V_j = D L^-H u, one eigenvector per CTA; the 128 threads own
 // rows (one warp per FP64 unit of the SM); reflectors and rows of L are staged in shared
-// memory.  A reflector step sums four warp partials through shared memory (double-buffered by
-// step parity, so one barrier per step); its elements are split into double-float pairs once, where
+// memory.  A reflector step sums four warp partials through shared memory (two sets, in turn over
+// the executed steps, so one barrier per step); its elements are split into double-float pairs once, where
 // they were staged (a split per use kept the FP64 unit busy with its predicated-off fallback).  The
 // triangular solve runs as in k_rr_trsm, from the last row up.
 template <int RPT>
@@ -1230,7 +1230,7 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
   double* sl = reinterpret_cast<double*>(stg + (size_t)scols * m);
   float2* stau = reinterpret_cast<float2*>(sl + m);               // tau as double-float pairs
   double* sdsc = sl + 2 * m;
-  __shared__ float4 red[8];    // warp partials of the reflector dot products, by step parity
+  __shared__ float4 red[8];    // warp partials of the reflector dot products, two sets in turn
   __shared__ double2 ysh[2];   // y_i of the triangular solve, by step parity
   const int tid = threadIdx.x, lane = tid & 31, wl = tid >> 5;
   const int j = blockIdx.x;
@@ -1258,6 +1258,8 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
       wq[q] = cdf0();
     }
   }
+  int set = 0;   // of the executed step: by the parity of k, two steps around an odd number of skipped
+                 // ones would share a set with no barrier between the reads and the writes
   for (int k1 = m - 3; k1 >= 0; k1 -= scols) {
     const int k0 = max(0, k1 - scols + 1);
     if (!stage_block(stg, cm + (size_t)k0 * m, (uint32_t)((k1 - k0 + 1) * m * sizeof(double2)), &mbar, phase)) {
@@ -1275,7 +1277,7 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
     __syncthreads();
     for (int k = k1; k >= k0; --k) {
       const dfl td{stau[k].x, stau[k].y};
-      if (td.h == 0.f) continue;   // uniform: every thread reads the same tau
+      if (td.h == 0.f) continue;   // no reflector (uniform: every thread reads the same tau), no barrier
       const float4* v = vdf + (size_t)(k - k0) * m;
       // rows r > k, thread-owned (r = tid + 128 q): partial dot, warp sums, four partials
       cdf sacc = cdf0();
@@ -1285,7 +1287,8 @@ __global__ void __launch_bounds__(128, 1) k_rr_backtr(double2* __restrict__ scr,
         if (r > k && r < m) sacc = cdf_fmac(ucdf(v[r]), wq[q], sacc);
       }
       sacc = warp_cdsum(sacc);
-      float4* part = red + 4 * (k & 1);
+      float4* part = red + 4 * set;
+      set ^= 1;
       if (lane == 0) part[wl] = c4(sacc);
       __syncthreads();
       const cdf tot = cadd(cadd(ucdf(part[0]), ucdf(part[1])), cadd(ucdf(part[2]), ucdf(part[3])));

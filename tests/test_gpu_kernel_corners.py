@@ -1,0 +1,50 @@
+"""Inputs that take a kernel off its common path: columns that need no reflector, blocks rotated in
+place, values near the ends of the FP32 range, planes that only just fit a block's shared memory."""
+import numpy as np
+import pytest
+
+from oracle import lobpcgf as olb
+
+from ._helpers import gpu, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _rand(shape, seed):
+    rng = np.random.default_rng(seed)
+    return rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
+
+
+# blocks of A on its diagonal: every block ends in two columns without a reflector and a 1 x 1 block
+# is one more, so that one, two and three (and longer runs of) steps are left out between executed ones
+@pytest.mark.parametrize("blocks", [(5, 1, 6, 1, 7), (40, 1, 39, 1, 1, 38), (2, 30, 2, 1, 64, 1, 1, 1, 29),
+                                    (1,) * 33, (100, 1, 60, 1, 139)])
+def test_rayleigh_ritz_decoupled_columns(blocks):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    nz = n = sum(blocks)
+    # one spectrum of even gaps dealt out to the blocks, so that no eigenvector is ill-conditioned
+    lam_all = np.random.default_rng(49).permutation(np.linspace(-3.0, 4.0, nz))
+    a, at = np.zeros((nz, nz), dtype=np.complex128), 0
+    for i, b in enumerate(blocks):
+        q = np.linalg.qr(_rand((b, b), 50 + i))[0]
+        h = (q * lam_all[at:at + b]) @ q.conj().T
+        a[at:at + b, at:at + b] = 0.5 * (h + h.conj().T)
+        at += b
+    s = np.eye(nz, dtype=np.complex128)
+    lam_ref, _, _ = olb.rayleigh_ritz(a, s, n)
+    # backward error of 2^-46 per operation and step of the double-float parts, |A| = 4: up to
+    # 4 nz 2^-46 |A| in the eigenvalues, the same over the gap in the vectors
+    tol = 4.0 * nz * 2.0 ** -46 * 4.0
+    gap = 7.0 / (nz - 1)
+    for _ in range(20):
+        v = torch.empty((n, nz), dtype=torch.complex128, device="cuda")
+        lam = torch.empty(n, dtype=torch.float64, device="cuda")
+        info = torch.zeros(4, dtype=torch.int32, device="cuda")
+        P.rayleigh_ritz(to_dev(a.T.copy(), torch.complex128), to_dev(s, torch.complex128), n, v, lam, info)
+        torch.cuda.synchronize()
+        assert info.cpu().numpy()[:3].tolist() == [0, nz, 0]
+        lg, vg = lam.cpu().numpy(), v.cpu().numpy().T
+        assert np.abs(lg - lam_ref).max() < tol
+        assert np.abs(vg.conj().T @ vg - np.eye(n)).max() < tol / gap
+        assert np.abs(a @ vg - vg * lg).max() < tol / gap
