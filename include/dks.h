@@ -352,7 +352,8 @@ int dks_tensor_cores_get(int* mask, int* kchunk);
 
 /* Algorithm 1's rotations (X <- Z V, P <- [0, Y, P] V): OUT[j] = sum_i Z[i] W[i + ldw*j] (+ beta OUT[j]) for
  * j < n, i < nz; Z [nz][rows], OUT [n][rows] (precision prec), W device
- * complex128 column-major with leading dimension ldw (converted to prec). */
+ * complex128 column-major with leading dimension ldw (converted to prec).  OUT does not overlap Z,
+ * except that OUT may be n <= 32 columns of Z itself (in place; W must not overlap OUT). */
 int dks_rotate(const void* Z, int rows, int nz, const void* W, int ldw, int n, void* OUT,
                double beta, int prec, void* stream);
 

@@ -452,15 +452,18 @@ int mirror_lower(double2* c, int m, cudaStream_t st) {
 // columns, 574 rows: 108 us with 64 x 32 tiles, which left 9 CTAs with 2.4 x the multiply-adds.)
 constexpr int ND_WARPS = 4;
 constexpr int ND_M = 64;   // inner indices staged at a time
+// In place (OUT overlaps A): a CTA holds RG = 2 x 32 rows of all n <= NI_COLS columns and writes after
+// a barrier, when nothing reads its rows any more.
+constexpr int NI_WARPS = 8, NI_NC = 4, NI_COLS = NI_WARPS * NI_NC;
 
-template <typename Va, typename Vo, int NC>
-__global__ void __launch_bounds__(32 * ND_WARPS) k_gemm_nn64(const Va* __restrict__ a, int lda, int k, int m,
-                                                             const double2* __restrict__ w, int ldw,
-                                                             const double* __restrict__ ws, int n,
-                                                             Vo* __restrict__ out, int ldo, double alpha, double beta) {
-  __shared__ double2 wsm[ND_WARPS * NC][ND_M];
-  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const int row = blockIdx.x * 32 + lane, cb = blockIdx.y * (ND_WARPS * NC), c0 = cb + wl * NC;
+template <typename Va, typename Vo, int NC, int NW = ND_WARPS, int RG = 1>
+__global__ void __launch_bounds__(32 * NW * RG) k_gemm_nn64(const Va* __restrict__ a, int lda, int k, int m,
+                                                            const double2* __restrict__ w, int ldw,
+                                                            const double* __restrict__ ws, int n,
+                                                            Vo* __restrict__ out, int ldo, double alpha, double beta) {
+  __shared__ double2 wsm[NW * NC][ND_M];
+  const int lane = threadIdx.x & 31, wl = (threadIdx.x >> 5) % NW, rg = (threadIdx.x >> 5) / NW;
+  const int row = (blockIdx.x * RG + rg) * 32 + lane, cb = blockIdx.y * (NW * NC), c0 = cb + wl * NC;
   const int nc = min(NC, n - c0);      // columns of this warp (none: it only helps staging W)
   double2 acc[NC];
 #pragma unroll
@@ -468,7 +471,7 @@ __global__ void __launch_bounds__(32 * ND_WARPS) k_gemm_nn64(const Va* __restric
   for (int m0 = 0; m0 < m; m0 += ND_M) {
     const int mn = min(ND_M, m - m0);
     __syncthreads();
-    for (int e = threadIdx.x; e < ND_WARPS * NC * ND_M; e += 32 * ND_WARPS) {
+    for (int e = threadIdx.x; e < NW * NC * ND_M; e += 32 * NW * RG) {
       const int mm = e & (ND_M - 1), cc = e / ND_M;
       double2 v{0, 0};
       if (mm < mn && cb + cc < n) {
@@ -490,6 +493,7 @@ __global__ void __launch_bounds__(32 * ND_WARPS) k_gemm_nn64(const Va* __restric
         if (j < nc) acc[j] = cfma(av, wsm[wl * NC + j][mm], acc[j]);
     }
   }
+  if constexpr (RG > 1) __syncthreads();   // in place: every read of the CTA's rows comes before the first write
   if (row >= k) return;
 #pragma unroll
   for (int j = 0; j < NC; ++j) {
@@ -658,6 +662,15 @@ int gemm_nn(const Va* a, int lda, int k, int m, const double2* w, int ldw, const
     }
     k_gemm_nn_f32<<<grid, 64 * g, NF_SMEM, st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, (float)beta);
   } else {
+    if constexpr (std::is_same<Va, Vo>::value) {
+      const Va *a1 = a + (size_t)std::max(0, m - 1) * lda + k, *o1 = out + (size_t)(n - 1) * ldo + k;
+      if (n <= NI_COLS && a < o1 && out < a1) {
+        k_gemm_nn64<Va, Vo, NI_NC, NI_WARPS, 2><<<(k + 63) / 64, 64 * NI_WARPS, 0, st>>>(a, lda, k, m, w, ldw, wscale, n,
+                                                                                        out, ldo, alpha, beta);
+        DKS_CUDA_TRY(cudaGetLastError());
+        return DKS_OK;
+      }
+    }
     const int rb = (k + 31) / 32;
     const long long warps = (long long)rb * n;
     auto grid = [&](int nc) { return dim3(rb, (n + ND_WARPS * nc - 1) / (ND_WARPS * nc)); };

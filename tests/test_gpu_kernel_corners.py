@@ -48,3 +48,29 @@ def test_rayleigh_ritz_decoupled_columns(blocks):
         assert np.abs(lg - lam_ref).max() < tol
         assert np.abs(vg.conj().T @ vg - np.eye(n)).max() < tol / gap
         assert np.abs(a @ vg - vg * lg).max() < tol / gap
+
+
+# up to 32 columns may be rotated into Z itself: around the 64 rows a block owns, the first columns
+# and the last ones, with and without beta
+@pytest.mark.parametrize("dtype", ["c64", "c128", "c128e"])
+@pytest.mark.parametrize("rows,nz,n,at,beta", [(1, 2, 2, 0, 0.0), (63, 5, 2, 3, 0.0), (64, 36, 5, 0, 0.5), (65, 36, 17, 19, 0.0),
+                                               (1500, 96, 32, 0, 0.0), (1500, 96, 32, 64, 2.0), (60000, 64, 31, 1, 0.0)])
+def test_rotate_in_place(rows, nz, n, at, beta, dtype):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    z0, w = _rand((nz, rows), 21), _rand((nz, n), 22)
+    z = to_dev(z0, torch.complex64 if dtype == "c64" else torch.complex128)
+    z0 = z.cpu().numpy().astype(np.complex128)
+    P.rotate(z, to_dev(w.T.copy(), torch.complex128), n, z[at:at + n], beta=beta, emulated=dtype == "c128e")
+    torch.cuda.synchronize()
+    got = z.cpu().numpy()
+    # rounding of nz + 2 products and sums each way: FP32, FP64, and the emulated form's 2^-48 of the
+    # largest value of each column
+    u = {"c64": 2.0 ** -24, "c128": 2.0 ** -53, "c128e": 2.0 ** -48}[dtype]
+    size = lambda a: np.abs(a.real) + np.abs(a.imag)  # noqa: E731
+    sz = size(z0) if dtype != "c128e" else np.broadcast_to(size(z0).max(axis=1, keepdims=True), z0.shape)
+    bound = (2 * nz + 8) * u * (size(w).T @ sz + abs(beta) * sz[at:at + n])
+    assert (np.abs(got[at:at + n] - (w.T @ z0 + beta * z0[at:at + n])) <= bound).all()
+    keep = np.ones(nz, dtype=bool)
+    keep[at:at + n] = False
+    assert np.array_equal(got[keep], z0[keep].astype(got.dtype))
