@@ -161,6 +161,17 @@ __device__ __forceinline__ double df_to_double(float h, float l, int k) {
   return __longlong_as_double(((long long)(hb >> 31) << 63) | (e << 52) | (m & ((1LL << 52) - 1)));
 }
 
+// the same for any pair: below 2^-63 (where the integer form drops a trailing part under 2^-126, and then
+// a leading part that is a subnormal number) and for infinities and NaN the sum is formed by the FP64
+// unit, out of line as in df_from_call
+static __device__ __noinline__ double df_val_call(float h, float l) { return (double)h + (double)l; }
+__device__ __forceinline__ double df_to_double_any(float h, float l) {
+  const unsigned hb = __float_as_uint(h);
+  const unsigned eh = (hb >> 23) & 255u;
+  if (eh >= 64u && eh < 255u) return df_to_double(h, l, 0);
+  return hb << 1 ? df_val_call(h, l) : 0.0;   // zero pairs are common (a zero block): no call
+}
+
 // complex double-float (16 bytes, the size of a double2)
 struct cdf {
   dfl re, im;

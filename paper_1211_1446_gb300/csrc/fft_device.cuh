@@ -144,7 +144,7 @@ __device__ __forceinline__ cdp cdp_split(double2 v) {
   return cdp{float2{re.h, im.h}, float2{re.l, im.l}};
 }
 __device__ __forceinline__ double2 to_d2(cdp v) {
-  return double2{df_to_double(v.h.x, v.l.x, 0), df_to_double(v.h.y, v.l.y, 0)};
+  return double2{df_to_double_any(v.h.x, v.l.x), df_to_double_any(v.h.y, v.l.y)};
 }
 template <typename V> __device__ __forceinline__ V vzero() { return V{0, 0}; }
 template <> __device__ __forceinline__ cdp vzero<cdp>() { return cdp{{0.f, 0.f}, {0.f, 0.f}}; }

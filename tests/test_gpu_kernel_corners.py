@@ -3,9 +3,10 @@ place, values near the ends of the FP32 range, planes that only just fit a block
 import numpy as np
 import pytest
 
+import workloads as W
 from oracle import lobpcgf as olb
 
-from ._helpers import gpu, to_dev
+from ._helpers import gpu, make_pair, rel_err, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -74,3 +75,23 @@ def test_rotate_in_place(rows, nz, n, at, beta, dtype):
     keep = np.ones(nz, dtype=bool)
     keep[at:at + n] = False
     assert np.array_equal(got[keep], z0[keep].astype(got.dtype))
+
+
+# H' is linear: a block scaled by a power of two gives the scaled result.  At 2^-100 the trailing parts
+# of the double-float values lie below the smallest normal FP32 number, 2^-126, and still count.
+@pytest.mark.parametrize("model", ["dks", "ksso"])
+@pytest.mark.parametrize("power", [0, 60, 93, 100])
+def test_emulated_h_small_scale(power, model):
+    torch = gpu()
+    nc = 4 if model == "dks" else 2
+    wl, ctx, hop, q = make_pair("small", model=model, projectors=False)
+    x = W.random_block(len(q), 3, 12, ncomp=nc)
+    if model == "dks":
+        x[:, 2:] = 0.0            # then the upper components of H' x are the local term alone
+    xd = to_dev(x * 2.0 ** -power, torch.complex128)
+    hx = torch.empty_like(xd)
+    ctx.apply_H(0, xd, hx, emulated=True)
+    torch.cuda.synchronize()
+    # the bound of the unscaled block: the granularity 2^-149 of FP32 is 2^-49 of a block of 2^-100, no more
+    # than the 2^-48 of a double-float step
+    assert rel_err(hx.cpu().numpy()[:, :2] * 2.0 ** power, hop(x)[:, :2]) < 1e-11
