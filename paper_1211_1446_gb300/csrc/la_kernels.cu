@@ -520,16 +520,21 @@ constexpr int NF_R = 256, NF_GMAX = 5, NF_CMAX = 8 * NF_GMAX, NF_M = 16;
 
 // Two shared-memory stages: the A chunk of the next 16 inner indices is copied with cp.async and
 // the W chunk fetched into registers while the current chunk is multiplied.
-constexpr size_t NF_SMEM = 2 * (size_t)NF_M * NF_R * sizeof(float2) + 2 * (size_t)NF_M * NF_CMAX * sizeof(float4);
+// They hold the G column groups of the CTA and no more, so that three CTAs of up to 16 columns fit an
+// SM: narrow outputs are bound by the loads in flight.  (229,676 rows, 40 -> 4 columns 37 us, 120 -> 16
+// 115; with stages of 40 columns, and so two CTAs, 58 and 155; the scalar form 45 and 143.)
+constexpr size_t nf_smem_bytes(int g) {
+  return 2 * (size_t)NF_M * (NF_R * sizeof(float2) + 8 * g * sizeof(float4));
+}
 
-__global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* __restrict__ a, int lda, int k, int m,
-                                                     const double2* __restrict__ w, int ldw,
-                                                     const double* __restrict__ ws, int n,
-                                                     float2* __restrict__ out, int ldo, double alpha, float beta) {
+template <int G>
+__global__ void __launch_bounds__(64 * (G <= 2 ? G : NF_GMAX), G <= 2 ? 3 : 2) k_gemm_nn_f32(
+    const float2* __restrict__ a, int lda, int k, int m, const double2* __restrict__ w, int ldw,
+    const double* __restrict__ ws, int n, float2* __restrict__ out, int ldo, double alpha, float beta) {
+  constexpr int T = 64 * G, ncols = 8 * G;
   extern __shared__ __align__(16) unsigned char nf_smem[];
   float2* as_base = reinterpret_cast<float2*>(nf_smem);                          // [2][NF_M][NF_R]
-  float4* ws_base = reinterpret_cast<float4*>(as_base + 2 * NF_M * NF_R);         // [2][NF_M][NF_CMAX]
-  const int ncols = (blockDim.x >> 6) * 8;
+  float4* ws_base = reinterpret_cast<float4*>(as_base + 2 * NF_M * NF_R);         // [2][NF_M][ncols]
   const int r0 = blockIdx.x * NF_R, c0 = blockIdx.y * ncols;
   const int rg = threadIdx.x & 63, cg = threadIdx.x >> 6;
   float2 acc[4][8];
@@ -539,7 +544,8 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
     for (int j = 0; j < 8; ++j) acc[i][j] = float2{0.f, 0.f};
   auto load_a = [&](int buf, int m0) {
     float2* dst = as_base + (size_t)buf * NF_M * NF_R;
-    for (int e = threadIdx.x; e < NF_M * NF_R; e += blockDim.x) {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < NF_M * NF_R; e += T) {
       const int rr = e & (NF_R - 1), mm = e >> 8;
       if (m0 + mm < m && r0 + rr < k) cp_async8(dst + e, a + (size_t)(m0 + mm) * lda + r0 + rr);
       else dst[e] = float2{0.f, 0.f};
@@ -550,7 +556,7 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
   auto fetch_w = [&](int m0, float2 (&wr)[2]) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      const int e = threadIdx.x + q * blockDim.x;
+      const int e = threadIdx.x + q * T;
       const int mm = e / ncols, cc = e - mm * ncols;
       float2 v{0.f, 0.f};
       if (m0 + mm < m && c0 + cc < n) {
@@ -562,12 +568,12 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
     }
   };
   auto store_w = [&](int buf, const float2 (&wr)[2]) {
-    float4* dst = ws_base + (size_t)buf * NF_M * NF_CMAX;
+    float4* dst = ws_base + (size_t)buf * NF_M * ncols;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      const int e = threadIdx.x + q * blockDim.x;
+      const int e = threadIdx.x + q * T;
       const int mm = e / ncols, cc = e - mm * ncols;
-      dst[mm * NF_CMAX + cc] = float4{wr[q].x, wr[q].y, -wr[q].y, wr[q].x};
+      dst[mm * ncols + cc] = float4{wr[q].x, wr[q].y, -wr[q].y, wr[q].x};
     }
   };
   const int nch = (m + NF_M - 1) / NF_M;
@@ -590,7 +596,7 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
     }
     __syncthreads();
     const float2* as = as_base + (size_t)cur * NF_M * NF_R;
-    const float4* wsm = ws_base + (size_t)cur * NF_M * NF_CMAX;
+    const float4* wsm = ws_base + (size_t)cur * NF_M * ncols;
 #pragma unroll 2
     for (int mm = 0; mm < NF_M; ++mm) {
       float2 av[4];
@@ -598,7 +604,7 @@ __global__ void __launch_bounds__(64 * NF_GMAX, 2) k_gemm_nn_f32(const float2* _
       for (int i = 0; i < 4; ++i) av[i] = as[mm * NF_R + rg + 64 * i];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const float4 wv = wsm[mm * NF_CMAX + cg * 8 + j];
+        const float4 wv = wsm[mm * ncols + cg * 8 + j];
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i][j] = cfma2(av[i], float2{wv.x, wv.y}, float2{wv.z, wv.w}, acc[i][j]);
       }
@@ -635,6 +641,11 @@ static int col_groups(int n, int maxg) {
   return std::max(1, (per + 7) / 8);
 }
 
+static auto nn_f32_for(int g) {
+  return g == 1 ? k_gemm_nn_f32<1> : g == 2 ? k_gemm_nn_f32<2> : g == 3 ? k_gemm_nn_f32<3>
+       : g == 4 ? k_gemm_nn_f32<4> : k_gemm_nn_f32<5>;
+}
+
 template <typename Va, typename Vo>
 int gemm_nn(const Va* a, int lda, int k, int m, const double2* w, int ldw, const double* wscale, int n,
             Vo* out, int ldo, double beta, cudaStream_t st, double alpha, int cat, int tc) {
@@ -656,11 +667,12 @@ int gemm_nn(const Va* a, int lda, int k, int m, const double2* w, int ldw, const
     dim3 grid((k + NF_R - 1) / NF_R, (n + NF_CMAX - 1) / NF_CMAX);
     static bool attr = false;
     if (!attr) {
-      DKS_CUDA_TRY(cudaFuncSetAttribute((const void*)k_gemm_nn_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)NF_SMEM));
+      for (int q = 1; q <= NF_GMAX; ++q)
+        DKS_CUDA_TRY(cudaFuncSetAttribute((const void*)nn_f32_for(q), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)nf_smem_bytes(q)));
       attr = true;
     }
-    k_gemm_nn_f32<<<grid, 64 * g, NF_SMEM, st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, (float)beta);
+    nn_f32_for(g)<<<grid, 64 * g, nf_smem_bytes(g), st>>>(a, lda, k, m, w, ldw, wscale, n, out, ldo, alpha, (float)beta);
   } else {
     if constexpr (std::is_same<Va, Vo>::value) {
       const Va *a1 = a + (size_t)std::max(0, m - 1) * lda + k, *o1 = out + (size_t)(n - 1) * ldo + k;

@@ -95,3 +95,21 @@ def test_emulated_h_small_scale(power, model):
     # the bound of the unscaled block: the granularity 2^-149 of FP32 is 2^-49 of a block of 2^-100, no more
     # than the 2^-48 of a double-float step
     assert rel_err(hx.cpu().numpy()[:, :2] * 2.0 ** power, hop(x)[:, :2]) < 1e-11
+
+
+# FP32 outputs of 1 to 5 groups of eight columns to a block, and of two and three blocks of them
+@pytest.mark.parametrize("n", [7, 15, 23, 24, 25, 31, 32, 33, 39, 47, 56, 65, 81])
+@pytest.mark.parametrize("rows", [3, 300])
+def test_rotate_fp32_widths(rows, n):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    nz = n + 10
+    z, w, o = _rand((nz, rows), 31).astype(np.complex64), _rand((nz, n), 32), _rand((n, rows), 33).astype(np.complex64)
+    out = to_dev(o, torch.complex64)
+    P.rotate(to_dev(z, torch.complex64), to_dev(w.T.copy(), torch.complex128), n, out, beta=1.0)
+    torch.cuda.synchronize()
+    z, o = z.astype(np.complex128), o.astype(np.complex128)
+    size = lambda a: np.abs(a.real) + np.abs(a.imag)  # noqa: E731
+    # one rounding of W, two per product and sum, one of the update
+    bound = (2 * nz + 6) * 2.0 ** -24 * (size(w).T @ size(z) + size(o))
+    assert (np.abs(out.cpu().numpy() - (w.T @ z + o)) <= bound).all()
