@@ -301,8 +301,12 @@ int dft3(dks_ctx* ctx, double2* g, bool fwd, cudaStream_t st) {
     int p = 1;   // the largest divisor of n that is at most its square root
     for (int d = 2; d * d <= n; ++d)
       if (n % d == 0) p = d;
-    // lines per CTA: about 384 outputs, three per thread
-    const int lines = (int)(ng / n), nl = std::max(1, 384 / n);
+    // lines per CTA: about 384 outputs, three per thread; where that leaves SMs without a CTA, as many
+    // lines as give each four (V_hxc on 16 x 15 x 18: 94 us, with 384 outputs 117, on 32 x 32 x 40 119 and
+    // 140; more CTAs on a larger grid cost more than they give: 48 x 48 x 48 205 against 187)
+    const int lines = (int)(ng / n);
+    int nl = std::max(1, 384 / n);
+    if (lines < nl * ctx->num_sms) nl = std::max(1, lines / (4 * ctx->num_sms));
     const size_t smem = (size_t)(2 * nl + 1) * n * sizeof(double2);
     Prof pr(P_SCF, st, 32.0 * ng, 8.0 * ng * (p + n / p + 1));
     k_dft_axis<<<(lines + nl - 1) / nl, 128, smem, st>>>(g, n1, n2, n3, axis, ctx->tw64[axis], fwd ? 1 : 0, p, nl,

@@ -113,3 +113,21 @@ def test_rotate_fp32_widths(rows, n):
     # one rounding of W, two per product and sum, one of the update
     bound = (2 * nz + 6) * 2.0 ** -24 * (size(w).T @ size(z) + size(o))
     assert (np.abs(out.cpu().numpy() - (w.T @ z + o)) <= bound).all()
+
+
+# grids of few lines (one or a few to a block) and of one line more or less than the blocks of a share
+@pytest.mark.parametrize("grid", [(12, 12, 12), (14, 12, 15), (24, 25, 27), (32, 32, 36), (36, 42, 35), (12, 12, 256)])
+def test_hxc_few_lines(grid):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    from oracle import scf as oscf
+    wl = W.make("small", grid=grid, ecut=1.0)
+    ctx = P.Context.from_workload(wl)
+    rho = np.random.default_rng(8).uniform(0.0, 0.1, grid)
+    v = torch.empty(grid, dtype=torch.float64, device="cuda")
+    eh, exc = ctx.hxc(to_dev(rho, torch.float64), v)
+    want, eh0, exc0 = oscf.hxc(rho, wl.lattice, wl.volume)
+    # at most 2 (p + q + 1) = 66 roundings of 2^-53 per axis and direction, six passes: 4.4e-14, and the
+    # reference's own
+    assert rel_err(v.cpu().numpy(), want) < 1e-13
+    assert abs(eh - eh0) < 1e-12 * abs(eh0) and abs(exc - exc0) < 1e-12 * abs(exc0)
