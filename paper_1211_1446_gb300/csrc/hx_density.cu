@@ -179,7 +179,7 @@ int density_accumulate(dks_ctx* ctx, int ik, const double2* x, int nb, const dou
         pr.count(1);
         const dim3 g1(n3, nf, (n1 + rpb - 1) / rpb);
         rows_inv<<<g1, 256, sm_r, st>>>(tbuf, pbuf, kp.nsticks, kp.stick_plane, e2, ld, n1, n3, ctx->etw64[1], rpb,
-                                        magic(rpb));
+                                        magic(rpb), magic(n1 - (n1 - 1) / rpb * rpb));
         const dim3 g2(n3, (n2 + cpb - 1) / cpb, (nf + fper - 1) / fper);
         cols_density<<<g2, 256, sm_cd, st>>>(pbuf, e1, ld, n2, n3, ctx->etw64[0], wf + (size_t)b0 * nc, nf, fper, cpb,
                                              ls1, magic(cpb), magic(n2 - (n2 - 1) / cpb * cpb), rho_perm);

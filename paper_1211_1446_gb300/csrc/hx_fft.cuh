@@ -180,14 +180,14 @@ template <typename Vs, bool BIG>
 __global__ void __launch_bounds__(256) k_plane_rows_inv(const Vs* __restrict__ t, Vs* __restrict__ pbuf, int nsticks,
                                                         const int* __restrict__ stick_plane, ExecPlan e2, int ld,
                                                         int n1, int n3, const typename TwOf<Vs>::T* __restrict__ tw2, int rpb,
-                                                        unsigned mrpb) {
+                                                        unsigned mrpb, unsigned mlast) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Vs* rows = reinterpret_cast<Vs*>(smem_raw);   // rpb rows of stride ld
   auto* tw = twiddle_space<Vs>(rows + rpb * ld);
   load_twiddles(tw, tw2, e2.ntw);
   const int z = blockIdx.x, f = blockIdx.y, r0 = blockIdx.z * rpb;
   const int nr = min(rpb, n1 - r0);
-  for (int e = threadIdx.x; e < rpb * ld; e += blockDim.x) rows[e] = vzero<Vs>();
+  for (int e = threadIdx.x; e < nr * ld; e += blockDim.x) rows[e] = vzero<Vs>();
   __syncthreads();
   const Vs* src = t + ((size_t)f * n3 + z) * nsticks;
   const int lo = r0 * ld, hi = (r0 + nr) * ld;   // stick_plane = i1 LD + i2
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256) k_plane_rows_inv(const Vs* __restrict__ t
     if (pos >= lo && pos < hi) rows[pos - lo] = src[s];
   }
   __syncthreads();
-  fft_axis<Vs, BIG>(rows, Lines{nullptr, ld, 1, rpb, mrpb}, e2, tw, false);   // rows beyond nr are zero
+  fft_axis<Vs, BIG>(rows, Lines{nullptr, ld, 1, nr, nr == rpb ? mrpb : mlast}, e2, tw, false);
   Vs* out = pbuf + (((size_t)f * n3 + z) * n1 + r0) * ld;
   for (int e = threadIdx.x; e < nr * ld; e += blockDim.x) out[e] = rows[e];
 }
@@ -516,7 +516,7 @@ int launch_plane(dks_ctx* ctx, const KPoint& kp, const ExecPlan& e1, const ExecP
     const unsigned mr = magic(rpb), mrl = magic(n1 - (n1 - 1) / rpb * rpb), mc = magic(cpb),
                    mcl = magic(n2 - (n2 - 1) / cpb * cpb);
     k_plane_rows_inv<Vs, BIG><<<g1, 256, sm_r, st>>>(tbuf, pbuf, kp.nsticks, kp.stick_plane, e2, ld, n1, n3, tw2,
-                                                         rpb, mr);
+                                                         rpb, mr, mrl);
     k_plane_cols_v<Vs, BIG><<<g2, 256, sm_cv, st>>>(pbuf, e1, ld, n2, n3, tw1, vp, cpb, ls1, mc, mcl);
     k_plane_rows_fwd<Vs, BIG><<<g1, 256, sm_r, st>>>(tbuf, pbuf, kp.nsticks, kp.stick_plane, e2, ld, n1, n3, tw2,
                                                          rpb, mr, mrl);

@@ -131,3 +131,25 @@ def test_hxc_few_lines(grid):
     # reference's own
     assert rel_err(v.cpu().numpy(), want) < 1e-13
     assert abs(eh - eh0) < 1e-12 * abs(eh0) and abs(exc - exc0) < 1e-12 * abs(exc0)
+
+
+# the row kernels of the split plane FFT take 40 (complex128) or 81 (complex64) rows to a block here: last
+# blocks of 1, 2, 3 and 4 rows, and a block that is not full
+@pytest.mark.parametrize("grid", [(81, 100, 12), (84, 100, 12), (42, 100, 12), (27, 100, 12)])
+@pytest.mark.parametrize("dtype", ["c64", "c128", "c128e"])
+def test_split_plane_last_rows(grid, dtype):
+    torch = gpu()
+    from oracle import scf as oscf
+    wl, ctx, hop, q = make_pair("small", grid=grid, ecut=4.0)
+    ctx.set_tuning(64 << 20, 0, 1)
+    x = W.random_block(len(q), 2, 13)
+    xd = to_dev(x, torch.complex64 if dtype == "c64" else torch.complex128)
+    hx = torch.empty_like(xd)
+    ctx.apply_H(0, xd, hx, emulated=dtype == "c128e")
+    torch.cuda.synchronize()
+    assert rel_err(hx.cpu().numpy(), hop(x)) < (2e-6 if dtype == "c64" else 1e-11)   # the operator's other tests
+    if dtype == "c128":
+        rho = torch.zeros(grid, dtype=torch.float64, device="cuda")
+        ctx.density(0, xd, [1.0, 0.5], rho)
+        torch.cuda.synchronize()
+        assert rel_err(rho.cpu().numpy(), oscf.density(x, ctx.basis(0), wl.grid, wl.volume, [1.0, 0.5])) < 1e-11
