@@ -159,6 +159,16 @@ struct dks_ctx {
 };
 
 namespace dks {
+// Pass B of H' in one kernel needs the whole N1 x LD plane in shared memory; larger planes (or a
+// tuner's choice, dks_ctx::plane_split) take the three-kernel form through the buffer P.
+constexpr size_t kPlaneSmem = 227 * 1024;
+inline bool plane_fits(const dks_ctx* ctx, size_t elem) {
+  return (size_t)ctx->grid[0] * ctx->plane_ld * elem <= kPlaneSmem;
+}
+inline bool split_plane(const dks_ctx* ctx, size_t elem) { return ctx->plane_split || !plane_fits(ctx, elem); }
+}  // namespace dks
+
+namespace dks {
 
 // ---------------------------------------------------------------- profiling
 enum ProfCat {

@@ -480,14 +480,4 @@ template <typename V>
 static size_t twiddle_bytes(int n) {
   return n * sizeof(typename TwOf<V>::T) + 16;
 }
-
-// Pass B in one kernel needs the whole N1 x LD plane in shared memory; larger planes (or a
-// tuner's choice, ctx->plane_split) take the three-kernel form through the buffer P.
-template <typename V>
-static bool split_plane(const dks_ctx* ctx) {
-  const ExecPlan* e = sizeof(V) == sizeof(float2) ? ctx->exec32 : ctx->exec64;
-  const size_t need = (size_t)ctx->grid[0] * ctx->plane_ld * sizeof(V) + twiddle_bytes<V>(e[0].ntw + e[1].ntw) +
-                      ctx->grid[0] * sizeof(int);
-  return ctx->plane_split || need > 227 * 1024;
-}
 }  // namespace dks

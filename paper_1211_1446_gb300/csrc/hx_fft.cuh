@@ -124,7 +124,10 @@ __host__ __device__ constexpr int plane_max_threads(size_t elem, bool big) {
 // (passes of axis 1) - 1 passes, the last inverse and the first forward pass of axis 1 and the
 // product with V being one.  Axis 2 runs over the rows that hold a stick only (29 of 60 for a grid
 // twice as fine as the sphere needs); the others are zero before and unused after.
-template <typename V, bool BIG>
+// TWS: the twiddles and the row table in shared memory after the plane; planes that leave no room for
+// them read both through L1, which beats the three-kernel form (4 columns, us: 160 x 180 x 12 complex64
+// 191 against 342, 120 x 120 x 12 double-float 301 against 360; 16 columns on 120 x 120 x 216 24.1 against 29.3 ms).
+template <typename V, bool BIG, bool TWS>
 __global__ void __launch_bounds__(plane_max_threads(sizeof(V), BIG), 1)
     k_plane(V* __restrict__ t, int nsticks, const int* __restrict__ stick_plane, const int* __restrict__ plane_rows,
             int nrows, unsigned mrows, const __grid_constant__ ExecPlan e1,
@@ -133,14 +136,21 @@ __global__ void __launch_bounds__(plane_max_threads(sizeof(V), BIG), 1)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* plane = reinterpret_cast<V*>(smem_raw);   // n1 rows of stride ld (odd), position i1*ld + i2
   const int np = e1.n * ld;
-  auto* stw1 = twiddle_space<V>(plane + np);
-  auto* stw2 = stw1 + e1.ntw;
-  int* rows = reinterpret_cast<int*>(stw2 + e2.ntw);
+  const typename TwOf<V>::T *ptw1 = tw1, *ptw2 = tw2;
+  const int* rows = plane_rows;
   const int z = blockIdx.x, f = blockIdx.y;
   for (int e = threadIdx.x; e < np; e += blockDim.x) plane[e] = vzero<V>();
-  load_twiddles(stw1, tw1, e1.ntw);
-  load_twiddles(stw2, tw2, e2.ntw);
-  for (int e = threadIdx.x; e < nrows; e += blockDim.x) rows[e] = plane_rows[e];
+  if constexpr (TWS) {
+    auto* stw1 = twiddle_space<V>(plane + np);
+    auto* stw2 = stw1 + e1.ntw;
+    int* srows = reinterpret_cast<int*>(stw2 + e2.ntw);
+    load_twiddles(stw1, tw1, e1.ntw);
+    load_twiddles(stw2, tw2, e2.ntw);
+    for (int e = threadIdx.x; e < nrows; e += blockDim.x) srows[e] = plane_rows[e];
+    ptw1 = stw1;
+    ptw2 = stw2;
+    rows = srows;
+  }
   __syncthreads();
   V* row = t + ((size_t)f * n3 + z) * nsticks;
   for (int s = threadIdx.x; s < nsticks; s += blockDim.x) {
@@ -157,7 +167,7 @@ __global__ void __launch_bounds__(plane_max_threads(sizeof(V), BIG), 1)
     const int k = i < a ? i : i < b ? i - a : i < c ? e1.nst - 2 - (i - b) : e2.nst - 1 - (i - c);
     const ExecPass& p = ax2 ? e2.p[k] : e1.p[k];
     const Lines ln{ax2 ? rows : nullptr, 1, ax2 ? 1 : ld, ax2 ? nrows : e2.n, ax2 ? mrows : mcols};
-    fft_step<V, BIG>(plane, ln, p, ax2 ? e2.n : e1.n, (ax2 ? stw2 : stw1) + p.tw, dit, i == b - 1 ? vz : nullptr);
+    fft_step<V, BIG>(plane, ln, p, ax2 ? e2.n : e1.n, (ax2 ? ptw2 : ptw1) + p.tw, dit, i == b - 1 ? vz : nullptr);
   }
   for (int s = threadIdx.x; s < nsticks; s += blockDim.x) {
     const int at = stick_plane[s];
@@ -498,13 +508,19 @@ int launch_stick_forward(dks_ctx* ctx, const KPoint& kp, const ExecPlan& e3, con
   return DKS_OK;
 }
 
+// shared memory of pass B in one kernel: the plane, its twiddles and its row table
+template <typename Vs>
+static size_t plane_smem(const dks_ctx* ctx, const KPoint& kp, const ExecPlan& e1, const ExecPlan& e2) {
+  return (size_t)e1.n * ctx->plane_ld * sizeof(Vs) + twiddle_bytes<Vs>(e1.ntw + e2.ntw) + kp.nrows * sizeof(int);
+}
+
 // pass B of nfi fields, in one kernel or split through pbuf
 template <typename Vs, bool BIG>
 int launch_plane(dks_ctx* ctx, const KPoint& kp, const ExecPlan& e1, const ExecPlan& e2,
                         const typename TwOf<Vs>::T* tw1, const typename TwOf<Vs>::T* tw2,
                         const typename RealOf<Vs>::T* vp, Vs* tbuf, Vs* pbuf, int nfi, cudaStream_t st) {
   const int n1 = e1.n, n2 = e2.n, n3 = ctx->grid[2], ld = ctx->plane_ld, ls1 = n1 | 1;
-  if (split_plane<Vs>(ctx)) {
+  if (split_plane(ctx, sizeof(Vs))) {
     if (!pbuf) return fail(DKS_ERR_INVALID_ARG, "split plane FFT without its buffer");
     const int rpb = lines_per_cta(n1, ld, sizeof(Vs)), cpb = lines_per_cta(n2, ls1, sizeof(Vs));
     const size_t sm_r = (size_t)rpb * ld * sizeof(Vs) + twiddle_bytes<Vs>(e2.ntw),
@@ -522,13 +538,29 @@ int launch_plane(dks_ctx* ctx, const KPoint& kp, const ExecPlan& e1, const ExecP
                                                          rpb, mr, mrl);
     return DKS_OK;
   }
-  const size_t sm = (size_t)n1 * ld * sizeof(Vs) + twiddle_bytes<Vs>(e1.ntw + e2.ntw) + kp.nrows * sizeof(int);
+  const size_t sm = plane_smem<Vs>(ctx, kp, e1, e2);
   const int tb = ctx->plane_threads > 0
                      ? ctx->plane_threads
                      : pick_plane_threads(e1, e2, kp.nrows, sm, plane_max_threads(sizeof(Vs), BIG));
-  DKS_TRY(allow_smem((const void*)k_plane<Vs, BIG>));
-  k_plane<Vs, BIG><<<dim3(n3, nfi), tb, sm, st>>>(tbuf, kp.nsticks, kp.stick_plane, kp.plane_rows, kp.nrows,
-                                                      magic(kp.nrows), e1, e2, ld, magic(n2), n3, tw1, tw2, vp);
+  DKS_TRY(allow_smem((const void*)k_plane<Vs, BIG, true>));
+  k_plane<Vs, BIG, true><<<dim3(n3, nfi), tb, sm, st>>>(tbuf, kp.nsticks, kp.stick_plane, kp.plane_rows, kp.nrows,
+                                                        magic(kp.nrows), e1, e2, ld, magic(n2), n3, tw1, tw2, vp);
+  return DKS_OK;
+}
+
+// pass B of planes that fit shared memory without their twiddles only
+template <typename Vs>
+int launch_plane_bare(dks_ctx* ctx, const KPoint& kp, const ExecPlan& e1, const ExecPlan& e2,
+                      const typename TwOf<Vs>::T* tw1, const typename TwOf<Vs>::T* tw2,
+                      const typename RealOf<Vs>::T* vp, Vs* tbuf, int nfi, cudaStream_t st) {
+  const int n3 = ctx->grid[2], ld = ctx->plane_ld;
+  const size_t sm = (size_t)e1.n * ld * sizeof(Vs);
+  const int tb = ctx->plane_threads > 0
+                     ? ctx->plane_threads
+                     : pick_plane_threads(e1, e2, kp.nrows, sm, plane_max_threads(sizeof(Vs), true));
+  DKS_TRY(allow_smem((const void*)k_plane<Vs, true, false>));
+  k_plane<Vs, true, false><<<dim3(n3, nfi), tb, sm, st>>>(tbuf, kp.nsticks, kp.stick_plane, kp.plane_rows, kp.nrows,
+                                                          magic(kp.nrows), e1, e2, ld, magic(e2.n), n3, tw1, tw2, vp);
   return DKS_OK;
 }
 
@@ -551,7 +583,7 @@ int fft_local(dks_ctx* ctx, const KPoint& kp, const Vg* x, Vg* out, int nb, int 
   const VR* vp = df ? (const VR*)ctx->vpermdf : fp64 ? (const VR*)ctx->vperm64 : (const VR*)ctx->vperm32;
   const int nc = ctx->ncomp;                   // fields per band: 4 (DKS) or 2 (KSSO)
   const int cat32 = fp64 ? 0 : kProf32;
-  const bool split = split_plane<Vs>(ctx);
+  const bool split = split_plane(ctx, sizeof(Vs));
   for (int b0 = 0; b0 < nb; b0 += chunk) {
     const int nbc = std::min(chunk, nb - b0);
     const Vg* xb = x + (size_t)b0 * nc * npw;
@@ -570,7 +602,9 @@ int fft_local(dks_ctx* ctx, const KPoint& kp, const Vg* x, Vg* out, int nb, int 
               nf * n3 * (10.0 * nn * std::log2(nn) + 2.0 * nn));
       if (split) pr.count(2);
       Vs* pbuf = reinterpret_cast<Vs*>(pbufv);
-      if (ep[0].big || ep[1].big)
+      if (!split && plane_smem<Vs>(ctx, kp, ep[0], ep[1]) > kPlaneSmem)
+        DKS_TRY((launch_plane_bare<Vs>(ctx, kp, ep[0], ep[1], tw1, tw2, vp, tbuf, nc * nbc, st)));
+      else if (ep[0].big || ep[1].big)
         DKS_TRY((launch_plane<Vs, true>(ctx, kp, ep[0], ep[1], tw1, tw2, vp, tbuf, pbuf, nc * nbc, st)));
       else
         DKS_TRY((launch_plane<Vs, false>(ctx, kp, ep[0], ep[1], tw1, tw2, vp, tbuf, pbuf, nc * nbc, st)));

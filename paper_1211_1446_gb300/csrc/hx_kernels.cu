@@ -132,10 +132,7 @@ int apply_h(dks_ctx* ctx, Exec& ex, int ik, const V* x, V* out, int nb, double s
   const size_t field_elems = (size_t)kp.nsticks * n3;
   // split pass B: one N1 x LD plane per (field, p3) in the buffer P (the arithmetic type of the
   // transforms has the size of V: complex128 and double-float pairs are both 16 bytes)
-  bool split = split_plane<V>(ctx);
-  if constexpr (std::is_same<V, double2>::value)
-    if (ex.df_gemm) split = split_plane<cdp>(ctx);
-  const size_t plane_elems = split ? (size_t)n3 * ctx->grid[0] * ctx->plane_ld : 0;
+  const size_t plane_elems = split_plane(ctx, sizeof(V)) ? (size_t)n3 * ctx->grid[0] * ctx->plane_ld : 0;
   // chunk of bands whose intermediates stay within the L2-resident budget
   int chunk = (int)std::max<size_t>(1, ctx->chunk_budget / (nc * (field_elems + plane_elems) * sizeof(V)));
   chunk = std::min(chunk, nb);

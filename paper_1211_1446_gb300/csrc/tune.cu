@@ -70,8 +70,7 @@ int dks_autotune(dks_ctx* ctx, int ik, int nb, int prec, void* stream, dks_tune_
   const size_t old_chunk = ctx->chunk_budget;
   const int old_threads = ctx->plane_threads, old_split = ctx->plane_split;
   // the one-kernel plane form is a candidate only where the plane fits one CTA
-  const size_t es_s = prec == DKS_PREC_FP32 ? sizeof(float2) : sizeof(double2);
-  const bool fits = (size_t)ctx->grid[0] * ctx->plane_ld * es_s <= 227 * 1024;
+  const bool fits = plane_fits(ctx, es);
   void* buf = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   DKS_CUDA_TRY(cudaMallocAsync(&buf, 2 * elems * es, st));

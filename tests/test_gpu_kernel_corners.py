@@ -153,3 +153,28 @@ def test_split_plane_last_rows(grid, dtype):
         ctx.density(0, xd, [1.0, 0.5], rho)
         torch.cuda.synchronize()
         assert rel_err(rho.cpu().numpy(), oscf.density(x, ctx.basis(0), wl.grid, wl.volume, [1.0, 0.5])) < 1e-11
+
+
+# planes whose data just fits a block's shared memory (227 KB), with room for the twiddles and without:
+# one kernel; one row or column more: three
+@pytest.mark.parametrize("grid,dtype,kernels", [((160, 180, 10), "c64", 1), ((168, 168, 10), "c64", 1),
+                                                ((168, 175, 10), "c64", 3), ((120, 120, 10), "c128", 1),
+                                                ((120, 120, 10), "c128e", 1), ((112, 125, 10), "c128e", 1),
+                                                ((125, 112, 10), "c128e", 1), ((90, 160, 10), "c128", 1),
+                                                ((120, 125, 10), "c128", 3), ((120, 125, 10), "c128e", 3)])
+def test_plane_at_the_shared_memory_limit(grid, dtype, kernels):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    wl, ctx, hop, q = make_pair("cubic", grid=grid, ecut=4.0)
+    x = W.random_block(len(q), 1, 14)
+    xd = to_dev(x, torch.complex64 if dtype == "c64" else torch.complex128)
+    want = hop(x)
+    for threads in (0, 64, 512):
+        ctx.set_tuning(64 << 20, threads, 0)
+        hx = torch.empty_like(xd)
+        P.profile_enable(True)
+        ctx.apply_H(0, xd, hx, emulated=dtype == "c128e")
+        count = P.profile_read()["plane_fft_v" + ("_fp32" if dtype == "c64" else "")]["launches"]
+        P.profile_enable(False)
+        assert count == kernels
+        assert rel_err(hx.cpu().numpy(), want) < (2e-6 if dtype == "c64" else 1e-11)   # the operator's other tests
