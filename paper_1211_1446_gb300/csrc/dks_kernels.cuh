@@ -41,18 +41,8 @@ __device__ __forceinline__ float2 cfma2(float2 a, float2 b, float2 ib, float2 c)
 }
 template <typename V>
 __device__ __forceinline__ V mul_i(V a) { return V{-a.y, a.x}; }
-template <typename V>
-__device__ __forceinline__ V mul_mi(V a) { return V{a.y, -a.x}; }
 template <typename V, typename T>
 __device__ __forceinline__ V cscale(V a, T s) { return V{a.x * s, a.y * s}; }
-
-// tw[t] = exp(+2 pi i t / N); forward transforms use the conjugate
-template <typename V>
-__device__ __forceinline__ V twiddle(const V* __restrict__ tw, int t, bool fwd) {
-  V w = __ldg(tw + t);
-  if (fwd) w.y = -w.y;
-  return w;
-}
 
 __device__ __forceinline__ double2 to_d2(double2 v) { return v; }
 __device__ __forceinline__ double2 to_d2(float2 v) { return double2{(double)v.x, (double)v.y}; }
@@ -183,24 +173,6 @@ __device__ __forceinline__ cdf csub(cdf a, cdf b) {
 __device__ __forceinline__ cdf cmul(cdf a, cdf b) {
   return cdf{df_add(df_mul(a.re, b.re), df_neg(df_mul(a.im, b.im))), df_add(df_mul(a.re, b.im), df_mul(a.im, b.re))};
 }
-__device__ __forceinline__ cdf mul_i(cdf a) { return cdf{df_neg(a.im), a.re}; }
-__device__ __forceinline__ cdf mul_mi(cdf a) { return cdf{a.im, df_neg(a.re)}; }
-__device__ __forceinline__ cdf cscale(cdf a, dfl s) { return cdf{df_mul(a.re, s), df_mul(a.im, s)}; }
-__device__ __forceinline__ cdf twiddle(const cdf* __restrict__ tw, int t, bool fwd) {
-  cdf w = tw[t];
-  if (fwd) w.im = df_neg(w.im);
-  return w;
-}
-__device__ __forceinline__ double2 to_d2(cdf v) { return double2{df_val(v.re), df_val(v.im)}; }
-template <> __device__ __forceinline__ cdf from_d2<cdf>(double2 v) { return cdf{df_from(v.x), df_from(v.y)}; }
-template <> struct RealOf<cdf> { using T = dfl; };
-
-// conversions between the storage type in global memory and the compute type in shared memory
-template <typename Vs> __device__ __forceinline__ Vs to_s(double2 v) { return from_d2<Vs>(v); }
-template <typename Vs> __device__ __forceinline__ Vs to_s(float2 v) { return v; }
-__device__ __forceinline__ double2 to_g(double2 v) { return v; }
-__device__ __forceinline__ float2 to_g(float2 v) { return v; }
-__device__ __forceinline__ double2 to_g(cdf v) { return to_d2(v); }
 
 // Index checks of the debug build (-DDKS_DEBUG, libdks_debug.so): a failed check records its code
 // in its translation unit's status word (the first failure is kept) and the caller skips the

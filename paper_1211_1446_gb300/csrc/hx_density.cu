@@ -166,8 +166,8 @@ int density_accumulate(dks_ctx* ctx, int ik, const double2* x, int nb, const dou
     {
       Prof pr(P_STICK_INV, st, (double)nf * npw * es + tb, 5.0 * n3 * std::log2((double)n3) * kp.nsticks * nf);
       const double2* xb = x + (size_t)b0 * nc * npw;
-      if (e3.big) DKS_TRY((launch_stick_inverse<double2, double2, true>(ctx, kp, e3, ctx->etw64[2], xb, tbuf, nf, st)));
-      else DKS_TRY((launch_stick_inverse<double2, double2, false>(ctx, kp, e3, ctx->etw64[2], xb, tbuf, nf, st)));
+      if (e3.big) DKS_TRY((launch_stick_inverse<double2, double2, true>(kp, e3, ctx->etw64[2], xb, tbuf, nf, st)));
+      else DKS_TRY((launch_stick_inverse<double2, double2, false>(kp, e3, ctx->etw64[2], xb, tbuf, nf, st)));
     }
     {
       // split the fields of a plane over enough CTAs to fill the GPU twice; atomics combine them

@@ -308,8 +308,7 @@ __device__ __forceinline__ void stick_lines_forward(const V* __restrict__ t, V* 
                                                     int lspb, int ls, unsigned mlines, const ExecPlan& e3,
                                                     const typename TwOf<V>::T* __restrict__ tw3) {
   auto* tw = twiddle_space<V>(line + ((NC * ls) << lspb));
-  load_twiddles(tw, tw3, e3.ntw);
-  if (e3.nst > 2) __syncthreads();   // the first DIT pass has no twiddles; its barrier publishes them
+  load_twiddles(tw, tw3, e3.ntw);   // the first DIT pass has none; the barrier after it publishes them
   fft_axis_load<V, BIG>(line, Lines{nullptr, ls, 1, NC << lspb, mlines}, e3, tw,
                         StickBuf<V>{const_cast<V*>(t) + s0, nsticks, ns, lspb, (size_t)e3.n * nsticks});
 }
@@ -477,7 +476,7 @@ static inline int lines_per_cta(int nlines, int line_stride, size_t elem, size_t
 }
 
 template <typename Vg, typename Vs, bool BIG3>
-int launch_stick_inverse(dks_ctx* ctx, const KPoint& kp, const ExecPlan& e3, const typename TwOf<Vs>::T* tw3, const Vg* x, Vs* t,
+int launch_stick_inverse(const KPoint& kp, const ExecPlan& e3, const typename TwOf<Vs>::T* tw3, const Vg* x, Vs* t,
                                 int nf, cudaStream_t st) {
   const int ls = e3.n | 1;                    // odd line stride: conflict-free shared memory
   const int l = pick_lspb(ls, sizeof(Vs), 1, 32 * 1024);
@@ -593,8 +592,8 @@ int fft_local(dks_ctx* ctx, const KPoint& kp, const Vg* x, Vg* out, int nb, int 
     const double f3 = 5.0 * n3 * std::log2((double)n3) * kp.nsticks * nf;
     {
       Prof pr(P_STICK_INV + cat32, st, nf * npw * es + tb, f3);
-      if (ep[2].big) DKS_TRY((launch_stick_inverse<Vg, Vs, true>(ctx, kp, ep[2], tw3, xb, tbuf, nc * nbc, st)));
-      else DKS_TRY((launch_stick_inverse<Vg, Vs, false>(ctx, kp, ep[2], tw3, xb, tbuf, nc * nbc, st)));
+      if (ep[2].big) DKS_TRY((launch_stick_inverse<Vg, Vs, true>(kp, ep[2], tw3, xb, tbuf, nc * nbc, st)));
+      else DKS_TRY((launch_stick_inverse<Vg, Vs, false>(kp, ep[2], tw3, xb, tbuf, nc * nbc, st)));
     }
     {
       const double nn = (double)ctx->grid[0] * ctx->grid[1];

@@ -394,6 +394,8 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
   // j+1, a warp elsewhere may still update with column j-1.
   // The update is bound by the FP64 unit (19 cycles of the SM per warp instruction): four fused
   // multiply-adds per element, on the lower triangle only.
+  // The columns in transit lie below the staging area: this bound asks for three columns of it more than
+  // the loop needs (m = 295 to 308 take the global form for that).
   const int ncol_own = (m + csize - 1) / csize;
   const bool dist = scols >= ncol_own + 3;
   for (size_t e = gtid; e < mm; e += gnt) {
@@ -479,7 +481,7 @@ __global__ void __launch_bounds__(RRC_THREADS, 1) k_rr_cluster(const double2* __
       RR_LAP(2);
     }
     if (failed) {
-      cl.sync();   // no CTA leaves while another may still read its published column
+      cl.sync();   // every CTA got here at the same column; none leaves before all have
     } else {
       // L_ij = lm_ij / sqrt(lm_jj) (i > j), L_jj = sqrt(lm_jj), and 1 / L_ii, from the owned columns
       double* linv = lamw + m;
@@ -1108,7 +1110,7 @@ __device__ __forceinline__ bool stage_wait(uint64_t* mbar, uint32_t parity, uint
 // stage `bytes` from src into dst (whole block); false (uniform over the block) on a timeout,
 // after a second bounded wait for the copy still in flight
 __device__ bool stage_block(void* dst, const void* src, uint32_t bytes, uint64_t* mbar, uint32_t& phase) {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier generic reads of dst
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier generic reads and writes of dst
   __syncthreads();
   if (threadIdx.x == 0) stage_issue(dst, src, bytes, mbar);
   const bool ok = __syncthreads_and(stage_wait(mbar, phase & 1, g_rr_first_wait) ? 1 : 0) != 0;
