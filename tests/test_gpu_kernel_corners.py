@@ -178,3 +178,51 @@ def test_plane_at_the_shared_memory_limit(grid, dtype, kernels):
         P.profile_enable(False)
         assert count == kernels
         assert rel_err(hx.cpu().numpy(), want) < (2e-6 if dtype == "c64" else 1e-11)   # the operator's other tests
+
+
+# pencils at which the Cholesky (295) and the Householder reduction (309) leave the staged form
+@pytest.mark.parametrize("nz", [294, 295, 308, 309])
+def test_rayleigh_ritz_staging_limits(nz):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    n = 20
+    z = _rand((nz, nz + 16), 41)
+    h = np.linspace(-3.0, 4.0, nz + 16)
+    a, s = (z * h) @ z.conj().T, z @ z.conj().T
+    lam_ref, _, info_ref = olb.rayleigh_ritz(a, s, n)
+    v = torch.empty((n, nz), dtype=torch.complex128, device="cuda")
+    lam = torch.empty(n, dtype=torch.float64, device="cuda")
+    info = torch.zeros(4, dtype=torch.int32, device="cuda")
+    P.rayleigh_ritz(to_dev(a.T.copy(), torch.complex128), to_dev(s.T.copy(), torch.complex128), n, v, lam, info)
+    torch.cuda.synchronize()
+    lam, v, info = lam.cpu().numpy(), v.cpu().numpy().T, info.cpu().numpy()
+    assert bool(info[0]) == info_ref.svqb and info[1] == info_ref.rank and info[2] == 0
+    # 2^-46 per operation of the double-float steps: nz 2^-46 |S^-1| |A|, |A| <= 4 |S|
+    tol = 4.0 * nz * 2.0 ** -46 * np.linalg.cond(s)
+    assert np.abs(lam - lam_ref).max() < 4.0 * tol
+    assert np.abs(v.conj().T @ s @ v - np.eye(n)).max() < tol
+    assert np.abs(a @ v - (s @ v) * lam).max() < 4.0 * tol * np.linalg.norm(s, 2) ** 0.5
+
+
+# complex64 Gram matrices sum 32 rows in FP32 and the rest in double-float pairs: the error stays that of
+# 32 rows however many there are (sums in FP32 throughout, or operands of fewer bits, are beyond it)
+@pytest.mark.parametrize("rows,nz", [(32, 17), (33, 31), (2060, 33), (20000, 40), (65537, 24)])
+def test_gram_fp32_folded_sums(rows, nz):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    z, hz = (to_dev(_rand((nz, rows), s), torch.complex64) for s in (61, 62))
+    a = torch.empty((nz, nz), dtype=torch.complex128, device="cuda")
+    s = torch.empty_like(a)
+    P.gram_hermitian(z, hz, a, s)
+    torch.cuda.synchronize()
+    z, hz = z.cpu().numpy().astype(np.complex128), hz.cpu().numpy().astype(np.complex128)
+    size = lambda x: np.abs(x.real) + np.abs(x.imag)  # noqa: E731
+    low = np.tril(np.ones((nz, nz), dtype=bool))
+    for got, b in ((a, hz), (s, z)):
+        err = np.abs(got.cpu().numpy().T - z.conj() @ b.T)
+        # two roundings of 2^-24 for each of at most 32 products of a part, and 2^-46 for every fold
+        bound = ((2 * min(rows, 32) + 4) * 2.0 ** -24 + (rows // 32 + 1) * 2.0 ** -46) * (size(z) @ size(b).T)
+        assert (err <= bound)[low].all()
+        # 64 steps of a part and chunk round independently by at most 2^-24 of a partial sum of RMS at most
+        # 8: 64 2^-24 for a chunk, both parts and rows / 32 chunks: 16 2^-24 sqrt(rows) off the diagonal
+        assert np.sqrt(np.mean(err[np.tril(low, -1)] ** 2)) < 16 * 2.0 ** -24 * np.sqrt(max(rows, 32))
