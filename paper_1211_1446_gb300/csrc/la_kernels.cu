@@ -48,8 +48,8 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // FP64 arithmetic (either operand complex128, or Acc64).  Bound by the FP64 unit: 1.7 fused
 // multiply-adds per clock and SM, so a warp's multiply-add takes 19 cycles of the whole SM and a
 // shared-memory operand per complex multiply-add is free beside it.  What counts is that every SM
-// has work and that none of it is padding: one output per thread, 16 x 16 tiles, and the k range
-// split until there are about four CTAs per SM.  (36 projector channels, 18 columns, 574 rows: 56 us
+// has work, to the end, and that none of it is padding: one output per thread, 16 x 16 tiles, and the
+// k range split into many CTAs per SM.  (36 projector channels, 18 columns, 574 rows: 56 us
 // with 48 x 32 tiles, whose 18 CTAs multiplied 2.4 x the outputs.)
 constexpr int HD_T = 16, HD_K = 32;
 
@@ -355,10 +355,26 @@ int gemm_hn(const Va* a, int lda, const Vb* b, int ldb, int k, int m, int n, dou
   const int tiles = lower ? mt * (mt + 1) / 2 : mt * nt;
   const int ktiles = (k + HN_T - 1) / HN_T;
   static_assert(HD_K == HN_T, "one k-tile length");
-  int splits = std::max(1, (4 * num_sms()) / tiles);
-  splits = std::min(splits, ktiles);
-  const int kchunk = ((ktiles + splits - 1) / splits) * HN_T;
-  splits = (k + kchunk - 1) / kchunk;
+  // k range split into chunks: about four CTAs per SM.  In FP64, where a k-tile takes about 9 us of an SM,
+  // 16, 12 or 4, whichever leaves the fullest SM fewest k-tiles, but no more than 4 x SMs chunks of one
+  // tile (their atomic additions meet in its 256 outputs).  (A^H B of 120 x 120, 57,419 rows: 13.1 ms with
+  // four CTAs per SM, 11.5 with 16; 48 x 48 1.77 with four, 1.75 with 12, 1.81 with 16; 4 x 4 57 us with
+  // four, 88 with 16.)
+  auto chunk_tiles = [&](int per_sm) {
+    const int s = std::min(std::min(std::max(1, per_sm * num_sms() / tiles), 4 * num_sms()), ktiles);
+    return (ktiles + s - 1) / s;
+  };
+  auto fullest = [&](int c) {
+    return ((long long)tiles * ((ktiles + c - 1) / c) + num_sms() - 1) / num_sms() * c;
+  };
+  int ct = chunk_tiles(acc32 ? 4 : 16);
+  if (!acc32)
+    for (int per_sm : {12, 4}) {
+      const int c = chunk_tiles(per_sm);
+      if (fullest(c) < fullest(ct)) ct = c;
+    }
+  const int kchunk = ct * HN_T;
+  const int splits = (k + kchunk - 1) / kchunk;
   dim3 grid(tiles, splits);
   const bool same = (const void*)a == (const void*)b;
   const bool f32 = sizeof(Va) == sizeof(float2) && sizeof(Vb) == sizeof(float2) && !Acc64;

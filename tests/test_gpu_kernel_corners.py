@@ -226,3 +226,23 @@ def test_gram_fp32_folded_sums(rows, nz):
         # 64 steps of a part and chunk round independently by at most 2^-24 of a partial sum of RMS at most
         # 8: 64 2^-24 for a chunk, both parts and rows / 32 chunks: 16 2^-24 sqrt(rows) off the diagonal
         assert np.sqrt(np.mean(err[np.tril(low, -1)] ** 2)) < 16 * 2.0 ** -24 * np.sqrt(max(rows, 32))
+
+
+# FP64 A^H B and its lower-triangle form with 12 and 16 blocks to an SM, last chunks of one row and of few
+@pytest.mark.parametrize("rows,nz", [(1, 3), (33, 96), (2060, 96), (2049, 17), (20001, 40), (57419, 48)])
+def test_gram_fp64_chunks(rows, nz):
+    torch = gpu()
+    import paper_1211_1446_gb300 as P
+    z, hz = (to_dev(_rand((nz, rows), s), torch.complex128) for s in (71, 72))
+    zn, hn = z.cpu().numpy(), hz.cpu().numpy()
+    size = lambda x: np.abs(x.real) + np.abs(x.imag)  # noqa: E731
+    low = np.tril(np.ones((nz, nz), dtype=bool))
+    for f, where in ((P.gram, np.ones((nz, nz), dtype=bool)), (P.gram_hermitian, low)):
+        a = torch.empty((nz, nz), dtype=torch.complex128, device="cuda")
+        s = torch.empty_like(a)
+        f(z, hz, a, s)
+        torch.cuda.synchronize()
+        for got, b in ((a, hn), (s, zn)):
+            err = np.abs(got.cpu().numpy().T - zn.conj() @ b.T)
+            # at most 2 rows + 4 roundings of 2^-53 on the way of any product, in the reference too
+            assert (err <= 2 * (2 * rows + 4) * 2.0 ** -53 * (size(zn) @ size(b).T))[where].all()
