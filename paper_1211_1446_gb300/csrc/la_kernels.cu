@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(32 * NW * RG) k_gemm_nn64(const Va* __restrict
 // over 256 rows and every shared-memory load of W feeds four complex multiply-adds.
 // Bound by issue: 50 % of the FMA pipe with scalar multiply-adds.  W lies in shared memory as
 // (w, i w), so that a complex multiply-add is two packed instructions (229,676 rows, 120 -> 40
-// columns: 258 -> 219 us, 40 TFLOP/s; the same bits).
+// columns: 258 -> 216 us, 41 TFLOP/s; the same bits).
 constexpr int NF_R = 256, NF_GMAX = 5, NF_CMAX = 8 * NF_GMAX, NF_M = 16;
 
 // Two shared-memory stages: the A chunk of the next 16 inner indices is copied with cp.async and
